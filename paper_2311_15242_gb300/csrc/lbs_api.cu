@@ -125,8 +125,31 @@ struct Layout {
 constexpr int kScal2 = 21, kScal3 = 25, kRest = 6;
 constexpr int kCoef2 = 6;  // 2D SOR coefficient planes (faces and inverse diagonals)
 constexpr int kNext2 = 5;  // 2D moments of t+1 written by the fused step (rho^R, rho^B, rho^N, j)
-// tile of the fused 2D step (k_lbfd2): TX x TY cells, one thread a cell
-constexpr int FTX = 32, FTY = 16;
+// tiles of the fused 2D step (k_lbfd2): TX x TY cells, one thread a cell
+struct FusedTile {
+    void *fn;
+    int tx, ty;
+    size_t smem;
+};
+template <typename R, typename P, int TX, int TY>
+FusedTile fused_tile() {
+    return {(void *)k_lbfd2<R, P, TX, TY>, TX, TY, Fuse2<R, TX, TY>::bytes()};
+}
+// 32 x 16, the least halo work a cell, or 16 x 8 where the larger tiles would
+// leave SMs idle.  FP64 is bound by the FP64 pipes of the SMs that have a
+// tile, one a SM: 16 x 8 wins up to one 32 x 16 tile an SM (128 x 128, 32
+// tiles: 309 -> 106 us; 250 x 250, 128: 311 -> 268; 300 x 400, 250: 428 -> 438).
+// FP32 is bound by the latency of a tile's phases, which a smaller tile
+// shortens while each still has an SM of its own, up to half the SMs (64 x
+// 517, 66 tiles: 22.1 -> 17.9 us; 64 x 1024, 128: 21.4 -> 19.9; 96 x 700,
+// 132: 20.0 -> 20.3; 128 x 1000, 252: 24.9 -> 25.9).
+template <typename R, typename P>
+FusedTile fused_tile_for(int nx, int ny, int sms) {
+    const FusedTile big = fused_tile<R, P, 32, 16>();
+    const long long tiles =
+        (long long)((nx + big.tx - 1) / big.tx) * ((ny + big.ty - 1) / big.ty);
+    return tiles <= (sizeof(R) == 8 ? sms : sms / 2) ? fused_tile<R, P, 16, 8>() : big;
+}
 
 template <typename R, typename P>
 Layout layout_of(const lbs_params *p) {
@@ -331,12 +354,16 @@ struct Solver : Base {
             cudaFuncSetAttribute(Launch3<R, P>::zm_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)Launch3<R, P>::zm_smem());
         if (D == 2) {
-            cudaFuncSetAttribute(k_lbfd2<R, P, FTX, FTY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)Fuse2<R, FTX, FTY>::bytes());
-            fgrid = dim3((p->nx + FTX - 1) / FTX, (p->ny + FTY - 1) / FTY, 1);
+            int dev = 0, sms = 1;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            ft = fused_tile_for<R, P>(p->nx, p->ny, sms);
+            cudaFuncSetAttribute(ft.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ft.smem);
+            fgrid = dim3((p->nx + ft.tx - 1) / ft.tx, (p->ny + ft.ty - 1) / ft.ty, 1);
         }
     }
-    dim3 fgrid;  // tiles of the fused 2D step
+    FusedTile ft = {};  // tile of the fused 2D step
+    dim3 fgrid;         // and its blocks
 
     // SOR variant: 2D the blocked tile (sor_vtx ...); 3D 0 = red-black
     // half-sweeps in place, 1 = z-marching full sweeps (ping-pong buffers),
@@ -542,7 +569,8 @@ struct Solver : Base {
             // the fused step: force, surfactant terms, collision, recolouring
             // and streaming in one launch (timed as the collide group) ...
             mark(s, LBS_K_COLLIDE);
-            k_lbfd2<R, P, FTX, FTY><<<fgrid, FTX * FTY, Fuse2<R, FTX, FTY>::bytes(), s>>>(I);
+            void *fargs[] = {(void *)&I};
+            CK(cudaLaunchKernel(ft.fn, fgrid, dim3(ft.tx * ft.ty), fargs, ft.smem, s));
             ran[LBS_K_COLLIDE] = true;
             if (I.transport && use_coop()) {
                 // ... then the gradient, every SOR round, the total and the
