@@ -264,7 +264,10 @@ int lbs_step_result(lbs_ctx *c, double *out);
  * are refused there).  More sweeps a launch mean fewer launches and a wider
  * halo (2 per sweep); the iterates, and so the results, do not depend on the
  * choice except through where the convergence test falls (after every
- * launch).  3D contexts: 0 = a red and a black half-sweep a sweep, in place,
+ * launch's sweeps).  With one launch a solve (lbs_set_sor_persistent) FP32 and
+ * 16-bit grids that fit the GPU at once take tiles chosen for their size instead
+ * (periodic x: even nx); the variant then sets the 2 or 4 sweeps between
+ * convergence tests.  3D contexts: 0 = a red and a black half-sweep a sweep, in place,
  * one thread a cell (default), 1 = one full red-black sweep a launch with
  * 32x8 tiles marching through 16-plane chunks of z in shared memory, 2 and
  * 3 = the half-sweeps of 0 with each thread marching a cell pair through 8
@@ -273,9 +276,10 @@ int lbs_set_sor_tile(lbs_ctx *c, int variant);
 
 /* 2D contexts: run the colour gradient at t+1, every round of a solve's
  * blocked SOR (Sec. 2.2), the total surfactant and the rescale in one
- * cooperative launch with grid barriers between them (on, the default; as
- * many blocks as are resident at once, each taking every gridsize-th tile of
- * a round), or the gradient, one launch a round inside the step graph's
+ * cooperative launch with grid barriers between them (on, the default; the
+ * whole grid resident at one tile a block where it fits, else as many blocks as
+ * are resident at once, each taking every gridsize-th tile of a round), or the
+ * gradient, one launch a round inside the step graph's
  * loop, the total and the rescale as launches of their own (off).  The
  * rounds are the same either way; the totals are summed in different
  * orders, so FP32 results agree to rounding.  In 3D the setting has no

@@ -17,6 +17,7 @@
 #include "lbs_internal.h"
 #include "lbs_k2d.cuh"
 #include "lbs_fused2.cuh"
+#include "lbs_solve2.cuh"
 #include "lbs_launch3.h"
 
 using namespace lbs;
@@ -72,6 +73,17 @@ size_t sor2_smem(int v) {
     }
 }
 #undef LBS_SORV
+
+// k_solve2 for K sweeps a round, NR rounds between grid barriers
+struct SolveForm {
+    int K, NR;
+    void *fn;
+    size_t smem;
+};
+template <int K, int NR>
+SolveForm solve_form() {
+    return {K, NR, (void *)k_solve2<K, NR>, SolveSmem<NR>::bytes};
+}
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -166,7 +178,10 @@ Layout layout_of(const lbs_params *p) {
     L.ctl_off = align_up(L.flag_off + 2 * (size_t)L.plane, 256);
     L.part_off = align_up(L.ctl_off + sizeof(Ctl), 256);
     L.nblocks = ((p->nx + BX - 1) / BX) * ((p->ny + BY - 1) / BY) * p->nz;
-    L.stage_off = align_up(L.part_off + (size_t)L.nblocks * (NDIAG + 3) * sizeof(double), 256);
+    // (reduction partials of a launch, or the records of k_solve2's blocks)
+    size_t part = (size_t)L.nblocks * (NDIAG + 3) * sizeof(double);
+    if (!d3 && part < kSolveRecBytes) part = kSolveRecBytes;
+    L.stage_off = align_up(L.part_off + part, 256);
     size_t N = (size_t)p->nx * p->ny * p->nz;
     L.total = align_up(L.stage_off + 12 * N * sizeof(double), 256);
     return L;
@@ -398,6 +413,29 @@ struct Solver : Base {
             const long long resident = (long long)per_sm * sms;
             coop_blocks = (int)(tiles < resident ? tiles : resident);
             coop_ok = coop && coop_blocks > 0;
+            set_solve(coop ? sms : 0);
+        }
+    }
+    // the grid resident on the chip (k_solve2): FP32 arithmetic, 2 or 4 sweeps
+    // a round and at most a tile an SM.  Two rounds of 2 sweeps between grid
+    // barriers where the wider halo's tiles still fit, else one.
+    SolveForm sf = {};
+    SolveGeom sg = {};
+    bool solve_ok = false;
+    void set_solve(int sms) {
+        solve_ok = false;
+        // (an odd periodic x axis would break the pairs of columns)
+        if (sizeof(R) != 4 || (!I.wall[0] && (I.nx & 1))) return;
+        const SolveForm f[] = {solve_form<2, 2>(), solve_form<2, 1>(), solve_form<4, 1>()};
+        for (const SolveForm &x : f) {
+            if (x.K != sor_vk(sv) || solve_ok) continue;
+            if (!solve_geom(I.nx, I.ny, I.wall, 2 * x.K * x.NR, sms, true, sg)) continue;
+            int per_sm = 0;
+            cudaFuncSetAttribute(x.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)x.smem);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, x.fn, kSolveThreads, x.smem);
+            if (per_sm < 1) continue;
+            sf = x;
+            solve_ok = true;
         }
     }
     int coop_blocks = 0;  // blocks of the one-launch form
@@ -446,6 +484,14 @@ struct Solver : Base {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         long long polls = coop_polls;
+        if (solve_ok) {
+            cfg.gridDim = dim3(sg.ntx * sg.nty, 1, 1);
+            cfg.blockDim = dim3(kSolveThreads, 1, 1);
+            cfg.dynamicSmemBytes = sf.smem;
+            void *args[] = {(void *)&I, (void *)&sg, (void *)&maxr, (void *)&polls};
+            CK(cudaLaunchKernelExC(&cfg, sf.fn, args));
+            return LBS_OK;
+        }
         void *args[] = {(void *)&I, (void *)&maxr, (void *)&polls};
         CK(cudaLaunchKernelExC(&cfg, sor2_coop_kernel<R>(sv), args));
         return LBS_OK;

@@ -295,11 +295,17 @@ __device__ __forceinline__ R two_sum(R a, R b, R &e) {
 // mirrored about the half-way wall (-1 -> 0, -2 -> 1, n -> n-1, ...).
 // refl: bit a set when axis a was reflected; side: -1 low wall, +1 high wall.
 // ---------------------------------------------------------------------------
+// (more than one period away: a call, which keeps its divisions out of the
+// callers' code)
+static __device__ __noinline__ int wrap_far(int c, int n) { return ((c % n) + n) % n; }
 __device__ __forceinline__ int map_axis(int c, int n, int wall, int bit, int &refl,
                                         int &side) {
     side = 0;
     if (c >= 0 && c < n) return c;
-    if (!wall) return ((c % n) + n) % n;
+    if (!wall) {
+        const int d = c < 0 ? c + n : c - n;
+        return d >= 0 && d < n ? d : wrap_far(c, n);
+    }
     refl |= bit;
     if (c < 0) {
         side = -1;
