@@ -103,3 +103,39 @@ def test_limit_of_rounds_and_restart():
     s.close()
     for k in a:
         assert np.array_equal(a[k], b[k]), k
+
+
+def test_gangs_of_a_batch_equal_single_contexts():
+    """Six instances whose tiles take two waves of the chip, one of odd height,
+    one taken out of the work lists: each as its own context, the inactive one
+    unchanged; and a batch with an odd periodic width, which the resident form
+    does not take."""
+    from paper_2311_15242_gb300 import Batch, Solver
+    cfgs = [W.bubble_rise_2d(nx=200 + 8 * k, ny=400 + (k == 2), D_b=32.0, Eo=2.0 + k)
+            for k in range(6)]
+    odd = droplet(nx=45, ny=40)
+    for group in (cfgs, [odd, cfgs[0]]):
+        fs = [W.initial_fields(c, seed=k, noise=0.02) for k, c in enumerate(group)]
+        b = Batch(group, storage="f32")
+        for k, f in enumerate(fs):
+            b.init_fields(k, f["phi"], f["psi"], f["C"], f["u"])
+        off = len(group) - 1
+        b.step(3)
+        kept = b.fields(off)
+        b.set_active(off, False)
+        b.step(9)
+        assert b.status() == [0] * len(group)
+        d = b.diagnostics()
+        for k, (c, f) in enumerate(zip(group, fs)):
+            got = b.fields(k)
+            if k == off:
+                assert all(np.array_equal(got[q], kept[q]) for q in got)
+                continue
+            s = Solver(c, storage="f32")
+            s.init_fields(f["phi"], f["psi"], f["C"], f["u"])
+            s.step(12)
+            err = errors(s.fields(), got)
+            assert within(err, F32_IMPL_TOL), (k, err)
+            assert s.diagnostics()["sor_iters_psi"] == d[k]["sor_iters_psi"]
+            s.close()
+        b.close()
