@@ -267,8 +267,9 @@ int lbs_step_result(lbs_ctx *c, double *out);
  * launch's sweeps).  With one launch a solve (lbs_set_sor_persistent) FP32 and
  * 16-bit grids that fit the GPU at once take tiles chosen for their size instead
  * (periodic x: even nx); the variant then sets the 2 or 4 sweeps between
- * convergence tests.  3D contexts: 0 = a red and a black half-sweep a sweep, in place,
- * one thread a cell (default), 1 = one full red-black sweep a launch with
+ * convergence tests.  3D contexts: 0 = a red and a black half-sweep a sweep, in
+ * place, one thread a cell, or the same sweeps in one launch a solve
+ * (lbs_set_sor_persistent) (default), 1 = one full red-black sweep a launch with
  * 32x8 tiles marching through 16-plane chunks of z in shared memory, 2 and
  * 3 = the half-sweeps of 0 with each thread marching a cell pair through 8
  * or 4 planes of z.  Errors: LBS_EINVAL. */
@@ -282,8 +283,9 @@ int lbs_set_sor_tile(lbs_ctx *c, int variant);
  * gradient, one launch a round inside the step graph's
  * loop, the total and the rescale as launches of their own (off).  The
  * rounds are the same either way; the totals are summed in different
- * orders, so FP32 results agree to rounding.  In 3D the setting has no
- * effect.  A barrier that waits too long (about a second) reports
+ * orders, so FP32 results agree to rounding.  3D contexts with SOR variant 0 in
+ * FP32 arithmetic: every sweep of a solve in one cooperative launch (on) or the
+ * half-sweeps as launches of their own (off): the same iterates.  A barrier that waits too long (about a second) reports
  * LBS_ETIMEOUT.  Errors: LBS_EINVAL (no context), LBS_ECUDA. */
 int lbs_set_sor_persistent(lbs_ctx *c, int on);
 

@@ -2,6 +2,7 @@
 // population storage forms (FP64, FP32, FP16 and bfloat16 with FP32 arithmetic).
 #include "lbs_k3d.cuh"
 #include "lbs_launch3.h"
+#include "lbs_sor3.cuh"
 
 namespace lbs {
 
@@ -93,6 +94,23 @@ int Launch3<R, P>::zm_threads() {
 template <typename R, typename P>
 size_t Launch3<R, P>::zm_smem() {
     return SorZm<R, kZmTX, kZmTY, kZmZC, kZmBS>::smem_bytes();
+}
+
+template <typename R, typename P>
+void *Launch3<R, P>::fs_fn() {
+    return sizeof(R) == 4 ? (void *)k_sor_fs3 : nullptr;
+}
+template <typename R, typename P>
+bool Launch3<R, P>::fs_geom(int nx, int ny, int nz, const int *wall, int blocks, Sor3Geom &g) {
+    return sor3_geom(nx, ny, nz, wall, blocks, g);
+}
+template <typename R, typename P>
+int Launch3<R, P>::fs_threads() {
+    return kSor3Threads;
+}
+template <typename R, typename P>
+size_t Launch3<R, P>::fs_smem() {
+    return kSor3Smem;
 }
 
 template struct Launch3<double, double>;

@@ -396,8 +396,22 @@ struct Solver : Base {
             // plane, or per chunk of planes when column marching)
             sor_grid = L3::sor_grid(sv, I.nx, I.ny, I.nz);
         }
-        I.sor_pingpong = (D == 2 || sv == 1) ? 1 : 0;
-        coop_ok = false;
+        coop_ok = fs_ok = false;
+        if (D == 3 && sv == 0 && L3::fs_fn()) {
+            // variant 0 in FP32 arithmetic: every sweep in one cooperative launch
+            int dev = 0, sms = 0, coop = 0, per_sm = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+            cudaFuncSetAttribute(L3::fs_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)L3::fs_smem());
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, L3::fs_fn(), L3::fs_threads(),
+                                                          L3::fs_smem());
+            fs_ok = coop && per_sm > 0 && L3::fs_geom(I.nx, I.ny, I.nz, I.wall, sms, fsg);
+            const long long tiles = (long long)fsg.ntx * fsg.nty * fsg.ntz;
+            fs_blocks = (int)(tiles < sms ? tiles : sms);
+        }
+        I.sor_pingpong = (D == 2 || sv == 1 || use_fs()) ? 1 : 0;
         if (D == 2) {
             // one launch for all rounds (k_sorfuse2): as many blocks as are
             // resident at once, up to one a tile; each block takes tiles b,
@@ -415,6 +429,28 @@ struct Solver : Base {
             coop_ok = coop && coop_blocks > 0;
             set_solve(coop ? sms : 0);
         }
+    }
+    // 3D: every sweep of a solve in one launch (k_sor_fs3) and its tiles
+    Sor3Geom fsg = {};
+    int fs_blocks = 0;
+    bool fs_ok = false;
+    bool use_fs() const { return D == 3 && fs_ok && coop_on; }
+    int launch_sor_fs(cudaStream_t s) {
+        int maxr = sor_rounds();
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(fs_blocks, 1, 1);
+        cfg.blockDim = dim3(L3::fs_threads(), 1, 1);
+        cfg.dynamicSmemBytes = L3::fs_smem();
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        long long polls = coop_polls;
+        void *args[] = {(void *)&I, (void *)&fsg, (void *)&maxr, (void *)&polls};
+        CK(cudaLaunchKernelExC(&cfg, L3::fs_fn(), args));
+        return LBS_OK;
     }
     // the grid resident on the chip (k_solve2): FP32 arithmetic, 2 or 4 sweeps
     // a round and at most a tile an SM.  Two rounds of 2 sweeps between grid
@@ -461,6 +497,7 @@ struct Solver : Base {
     int set_sor_persistent(int on) override {
         CK(cudaStreamSynchronize(ctx->stream));
         coop_on = on != 0;
+        if (D == 3) set_sor_grid();
         if (gexec) {
             CK(cudaGraphExecDestroy(gexec));
             CK(cudaGraphDestroy(graph));
@@ -653,7 +690,11 @@ struct Solver : Base {
             ran[LBS_K_GRAD] = true;
         }
         mark(s, LBS_K_SOR);
-        if (I.transport && !capturing) {
+        if (I.transport && use_fs()) {
+            int r = launch_sor_fs(s);
+            if (r) return r;
+            ran[LBS_K_SOR] = true;
+        } else if (I.transport && !capturing) {
             // eager form (for profilers): the host reads the loop state after
             // every round and launches no round beyond the converged one
             for (int r = 0; r < sor_rounds(); r++) {
@@ -948,6 +989,7 @@ struct Solver : Base {
     // red-black half-sweeps
     int kernel_count() const override {
         if (D == 2 && I.transport && use_coop()) return 2;
+        if (use_fs()) return I.transport ? 8 : 6;
         const int per_round = (D == 3 && sv != 1) ? 2 : 1;
         const int cells = D == 2 ? 2 : 5;  // 2D: the fused step and the gradient
         return I.transport ? cells + 2 + per_round * last_rounds : cells + 1;

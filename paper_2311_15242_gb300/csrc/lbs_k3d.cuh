@@ -129,6 +129,10 @@ __global__ void k_moments3(Inst<R> I) {
 // colour fraction that is small on the cell's side (see k_grad2)
 template <typename R>
 __global__ void k_grad3(Inst<R> I, int guess = 1) {
+    // (the one-launch SOR that follows starts from a clear barrier)
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 &&
+        threadIdx.y == 0)
+        I.ctl->bar_count = 0;
     LBS_CELL3
     const bool blue_side = I.rhoN[c] <= R(0);
     const Ax X = make_ax(x, I.nx, I.wall[0], 1), Y = make_ax(y, I.ny, I.wall[1], 2),

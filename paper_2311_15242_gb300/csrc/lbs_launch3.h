@@ -9,6 +9,14 @@
 
 namespace lbs {
 
+// tiles of k_sor_fs3 (lbs_sor3.cuh): their numbers, sizes (see solve_axis; tz
+// even) and the outer tiles' extra columns and rows
+struct Sor3Geom {
+    int ntx, nty, ntz;
+    int tx, ty, tz;
+    int ex, ey;
+};
+
 template <typename R, typename P>
 struct Launch3 {
     static void init(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s, const double *phi,
@@ -38,6 +46,13 @@ struct Launch3 {
     static dim3 zm_grid(int nx, int ny, int nz);
     static int zm_threads();
     static size_t zm_smem();
+    // every sweep of a solve in one cooperative launch (k_sor_fs3, FP32
+    // arithmetic; nullptr: none): kernel, tiles and threads of a grid for
+    // `blocks` blocks, shared memory
+    static void *fs_fn();
+    static bool fs_geom(int nx, int ny, int nz, const int *wall, int blocks, Sor3Geom &g);
+    static int fs_threads();
+    static size_t fs_smem();
 };
 
 }  // namespace lbs

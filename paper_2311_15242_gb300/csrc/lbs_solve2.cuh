@@ -58,12 +58,13 @@ struct __align__(16) SolveRec {
 };
 constexpr size_t kSolveRecBytes = 2 * (size_t)kSolveMaxBlocks * sizeof(SolveRec);
 
-// tile side and number of tiles along an axis: n cells, `walled` ends,
-// at most `most` tiles; the smallest number of tiles >= least that fits the
+// tile side and number of tiles along an axis: n cells, `walled` ends, halo H,
+// regions of at most `region` cells, at most `most` tiles; the smallest number of tiles >= least that fits the
 // region; false if none does
-inline bool solve_axis(int n, bool walled, int H, int least, int most, int &nt, int &t, int &e) {
+inline bool solve_axis(int n, bool walled, int H, int region, int least, int most, int &nt, int &t,
+                       int &e) {
     e = walled ? H : 0;
-    const int inner = kSolveRegion - 2 * H;
+    const int inner = region - 2 * H;
     for (int want = least < 1 ? 1 : least; want <= most; want++) {
         const int m = n - 2 * e;
         nt = want;
@@ -72,7 +73,7 @@ inline bool solve_axis(int n, bool walled, int H, int least, int most, int &nt, 
         while (nt > 1 && e + (nt - 1) * t >= n) nt--;  // (rounding up left a tile empty)
         if (nt == 1) {
             t = n + (n & 1);
-            if (walled ? n <= kSolveRegion : t <= inner) return true;
+            if (walled ? n <= region : t <= inner) return true;
         } else if (t <= inner && n - e - (nt - 1) * t <= inner + (walled ? H : 0)) {
             return true;
         }
@@ -87,14 +88,14 @@ inline bool solve_axis(int n, bool walled, int H, int least, int most, int &nt, 
 inline bool solve_geom(int nx, int ny, const int *wall, int H, int blocks, bool small,
                        SolveGeom &g) {
     if (blocks > kSolveMaxBlocks) blocks = kSolveMaxBlocks;
-    if (!solve_axis(nx, wall[0] != 0, H, 1, blocks, g.ntx, g.tx, g.ex)) return false;
+    if (!solve_axis(nx, wall[0] != 0, H, kSolveRegion, 1, blocks, g.ntx, g.tx, g.ex)) return false;
     const int most = blocks / g.ntx;
     int least = 1;
     if (small) {
         least = (ny + 15) / 16;
         if (least > most) least = most;
     }
-    return solve_axis(ny, wall[1] != 0, H, least, most, g.nty, g.ty, g.ey) &&
+    return solve_axis(ny, wall[1] != 0, H, kSolveRegion, least, most, g.nty, g.ty, g.ey) &&
            (long long)g.ntx * g.nty <= blocks;
 }
 
