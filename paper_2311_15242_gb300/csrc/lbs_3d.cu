@@ -18,12 +18,12 @@ void Launch3<R, P>::moments(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s) {
     k_moments3<R, P><<<g, b, 0, s>>>(I);
 }
 template <typename R, typename P>
-void Launch3<R, P>::grad(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s, int guess) {
-    k_grad3<R><<<g, b, 0, s>>>(I, guess);
+void Launch3<R, P>::grad(const Inst<R> &I, cudaStream_t s, int guess) {
+    k_grad3<R><<<tile3_grid(I), Tile3<R>::NT, 0, s>>>(I, guess);
 }
 template <typename R, typename P>
-void Launch3<R, P>::force(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s) {
-    k_force3<R><<<g, b, 0, s>>>(I);
+void Launch3<R, P>::force(const Inst<R> &I, cudaStream_t s) {
+    k_force3<R><<<tile3_grid(I), Tile3<R>::NT, 0, s>>>(I);
 }
 template <typename R, typename P>
 void Launch3<R, P>::fd(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s, double *Sout,
@@ -31,8 +31,8 @@ void Launch3<R, P>::fd(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s, double 
     k_fd3<R><<<g, b, 0, s>>>(I, Sout, Bout);
 }
 template <typename R, typename P>
-void Launch3<R, P>::collide(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s) {
-    k_collide3<R, P><<<g, b, 0, s>>>(I);
+void Launch3<R, P>::collide(const Inst<R> &I, cudaStream_t s) {
+    k_collide3<R, P><<<tile3_grid(I), Tile3<R>::NT, 0, s>>>(I);
 }
 template <typename R, typename P>
 void Launch3<R, P>::stream(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s) {

@@ -622,7 +622,7 @@ struct Solver : Base {
         if (D == 2)
             k_force2<R><<<grid, block, 0, s>>>(I);
         else
-            L3::force(I, grid, block, s);
+            L3::force(I, s);
     }
 
     // a kernel that directly follows another kernel of the step (no event or
@@ -680,13 +680,13 @@ struct Solver : Base {
                 ran[LBS_K_FD] = true;
             }
             mark(s, LBS_K_COLLIDE);
-            L3::collide(I, grid, block, s);
+            L3::collide(I, s);
             ran[LBS_K_COLLIDE] = true;
             mark(s, LBS_K_STREAM);
             L3::stream(I, grid, block, s);
             ran[LBS_K_STREAM] = true;
             mark(s, LBS_K_GRAD);
-            L3::grad(I, grid, block, s);
+            L3::grad(I, s);
             ran[LBS_K_GRAD] = true;
         }
         mark(s, LBS_K_SOR);
@@ -1046,7 +1046,7 @@ struct Solver : Base {
             L3::init(I, grid, block, s, dphi, psi ? dpsi : nullptr, C ? dC : nullptr,
                      u ? du : nullptr);
             L3::moments(I, grid, block, s);
-            L3::grad(I, grid, block, s, 0);
+            L3::grad(I, s, 0);
         }
         k_surf2<R, BS><<<surf_grid, block, 0, s>>>(I, 0, surf_blocks, sweeps_per_round());
         int r = launch_check();

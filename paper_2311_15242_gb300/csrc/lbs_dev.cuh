@@ -342,16 +342,23 @@ __device__ __forceinline__ long long nbx2(const Inst<R> &I, const Ax &X, const A
     sy = Y.s[dy + 2];
     return (long long)Y.v[dy + 2] * I.pitch + X.v[dx + 2];
 }
+// cell (x, y, z) of a 3D grid in 32 bits (a plane of 2^32 cells would be a
+// terabyte of state): one widening multiply-add an address instead of 64-bit
+// index arithmetic
+template <typename R>
+__device__ __forceinline__ unsigned icell3(const Inst<R> &I, int x, int y, int z) {
+    return ((unsigned)z * I.ny + y) * I.pitch + x;
+}
 // neighbour (dx, dy, dz) of a 3D cell from its axes
 template <typename R>
-__device__ __forceinline__ long long nbx3(const Inst<R> &I, const Ax &X, const Ax &Y, const Ax &Z,
-                                          int dx, int dy, int dz, int &refl, int &sx, int &sy,
-                                          int &sz) {
+__device__ __forceinline__ unsigned nbx3(const Inst<R> &I, const Ax &X, const Ax &Y, const Ax &Z,
+                                         int dx, int dy, int dz, int &refl, int &sx, int &sy,
+                                         int &sz) {
     refl = X.r[dx + 2] | Y.r[dy + 2] | Z.r[dz + 2];
     sx = X.s[dx + 2];
     sy = Y.s[dy + 2];
     sz = Z.s[dz + 2];
-    return ((long long)Z.v[dz + 2] * I.ny + Y.v[dy + 2]) * I.pitch + X.v[dx + 2];
+    return icell3(I, X.v[dx + 2], Y.v[dy + 2], Z.v[dz + 2]);
 }
 
 // programmatic dependent launch.  A kernel launched as the programmatic

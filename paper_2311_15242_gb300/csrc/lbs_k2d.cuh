@@ -360,31 +360,26 @@ __global__ void k_force2(Inst<R> I) {
 //   rhs_psi = w psi + (Ds/2) L_w psi + {S (t = 0) | 3/2 S - 1/2 S_prev}
 //   with w = a + eps_w and L_w the flux-form operator of Eq. 28.
 // ---------------------------------------------------------------------------
+// (the difference from the low side, `up`: over v[-2..1], or the high one,
+// over v[-1..2]; both are the same arithmetic on mirrored nodes, so the side is
+// a choice of operands, not of code)
 template <typename R>
-__device__ __forceinline__ R weno_m(const R *v) {  // v points at node i, v[-2..1]
+__device__ __forceinline__ R weno(const R *v, bool up) {  // v points at node i
     const R eps = R(1e-6);
-    R d2m = v[0] - R(2) * v[-1] + v[-2];
-    R d20 = v[1] - R(2) * v[0] + v[-1];
-    R r = fdiv(eps + d2m * d2m, eps + d20 * d20);
-    R w = fdiv(R(1), R(1) + R(2) * r * r);
-    R dpm2 = v[-1] - v[-2], dpm1 = v[0] - v[-1], dp0 = v[1] - v[0];
-    return R(0.5) * ((dpm1 + dp0) - w * (dpm2 - R(2) * dpm1 + dp0));
-}
-template <typename R>
-__device__ __forceinline__ R weno_p(const R *v) {  // v[-1..2]
-    const R eps = R(1e-6);
-    R d2p = v[2] - R(2) * v[1] + v[0];
-    R d20 = v[1] - R(2) * v[0] + v[-1];
-    R r = fdiv(eps + d2p * d2p, eps + d20 * d20);
-    R w = fdiv(R(1), R(1) + R(2) * r * r);
-    R dpm1 = v[0] - v[-1], dp0 = v[1] - v[0], dp1 = v[2] - v[1];
-    return R(0.5) * ((dpm1 + dp0) - w * (dp1 - R(2) * dp0 + dpm1));
+    const R b = up ? v[-1] : v[1], e = up ? v[-2] : v[2];
+    const R d2 = (up ? v[0] : e) - R(2) * b + (up ? e : v[0]);
+    const R d20 = v[1] - R(2) * v[0] + v[-1];
+    const R r = fdiv(eps + d2 * d2, eps + d20 * d20);
+    const R w = fdiv(R(1), R(1) + R(2) * r * r);
+    const R dm = v[0] - v[-1], dp = v[1] - v[0];
+    const R far = up ? b - e : e - b;
+    return R(0.5) * ((dm + dp) - w * (far - R(2) * (up ? dm : dp) + (up ? dp : dm)));
 }
 template <typename R>
 __device__ __forceinline__ R upwind(const R *v, R u) {
-    if (u > R(0)) return weno_m(v);
-    if (u < R(0)) return weno_p(v);
-    return R(0.5) * (weno_m(v) + weno_p(v));
+    const R d = weno(v, u > R(0));
+    if (u > R(0) || u < R(0)) return d;
+    return R(0.5) * (weno(v, true) + d);
 }
 
 // Sout, Bout: when given, only S and B of the current state are written

@@ -71,7 +71,7 @@ __device__ __forceinline__ void store_moments3(const Inst<R> &I, long long c, co
     const int y = blockIdx.y * blockDim.y + threadIdx.y;        \
     const int z = blockIdx.z;                                   \
     if (x >= I.nx || y >= I.ny) return;                         \
-    const long long c = cell3(I, x, y, z);
+    const unsigned c = icell3(I, x, y, z);
 
 // initial populations f^k = M^{-1} m^{k,eq}(rho^k, u) (Eq. 40), in double
 // precision and rounded once.  Inputs: dense double arrays [nz][ny][nx].
@@ -125,64 +125,153 @@ __global__ void k_moments3(Inst<R> I) {
     store_moments3(I, c, fT, fM, I.flag[c]);
 }
 
+// ---------------------------------------------------------------------------
+// Tiles of the stencil kernels (k_grad3, k_force3, k_collide3): a block of 256
+// threads owns 16 x 8 x TZ cells and keeps what the 18-point stencils read,
+// with a halo of one cell, in shared memory.  Those kernels are bound by
+// instruction issue: a cell that gathers its neighbours itself maps, wraps and
+// transforms (normal, colour fraction, ghost velocity) each of them 18 times
+// over; a tile does so once a slot, 2.1 slots a cell, and the stencil is left
+// with a shared load at a constant offset and its arithmetic (force: 1050 -> 420
+// warp instructions for 32 cells, collision 2600 -> 1700).
+// A thread fills one column of slots (its x and y mapped once) and owns TZ / 2
+// cells: a warp covers 16 cells of a row on two planes, so a grid that is no
+// multiple of 32 wide wastes fewer lanes than with rows of 32, and planes are
+// 16 banks apart (stride 208), which keeps both halves of the warp off each
+// other's banks.  4 planes a tile rather than 8: half the shared memory and
+// twice the blocks (force 35 -> 29 us, collision 111 -> 102 at 100 cubed,
+// although a cell then reads 2.1 slots instead of 1.8); FP64 takes 2 to stay
+// within 48 KB.  Measured in FP32 at 100 cubed: gradient 34 -> 25 us, force 57
+// -> 29, collision 129 -> 103; at 256 x 128 x 128 with BF16 populations 88 -> 66,
+// 226 -> 165, 406 -> 304.  What is left is the wait for memory: 25 to 60 % of
+// the issue slots are used, 20 to 55 % of the copy bandwidth.
+// ---------------------------------------------------------------------------
+template <typename R>
+struct Tile3 {
+    static constexpr int TX = 16, TY = 8, TZ = sizeof(R) == 4 ? 4 : 2;
+    static constexpr int HX = TX + 2, HY = TY + 2, PS = 208, N = (TZ + 2) * PS;
+    static constexpr int NT = 256;
+    static_assert(HX * HY <= PS && HX * HY <= NT && TX * TY * 2 == NT, "");
+    __host__ __device__ static constexpr int off(int dx, int dy, int dz) {
+        return dz * PS + dy * HX + dx;
+    }
+};
+template <typename R>
+inline dim3 tile3_grid(const Inst<R> &I) {
+    using T = Tile3<R>;
+    return dim3((I.nx + T::TX - 1) / T::TX, (I.ny + T::TY - 1) / T::TY, (I.nz + T::TZ - 1) / T::TZ);
+}
+
+// calls f(slot, cell, refl, sx, sy, sz) for every slot of the block's tile and
+// halo that the stencils of its cells read (refl, s*: as nbx3).  A slot further
+// out (past the end of the grid by more than the halo) gets some cell.
+template <typename R, typename F>
+__device__ __forceinline__ void tile3_fill(const Inst<R> &I, F &&f) {
+    using T = Tile3<R>;
+    const int t = threadIdx.x;
+    if (t >= T::HX * T::HY) return;
+    int rxy = 0, sx, sy;
+    int X = map_axis(int(blockIdx.x) * T::TX + t % T::HX - 1, I.nx, I.wall[0], 1, rxy, sx);
+    int Y = map_axis(int(blockIdx.y) * T::TY + t / T::HX - 1, I.ny, I.wall[1], 2, rxy, sy);
+    X = max(X, 0);  // (a mirror image further out than the axis is long)
+    Y = max(Y, 0);
+    const int z0 = int(blockIdx.z) * T::TZ;
+#pragma unroll 5
+    for (int k = 0; k < T::TZ + 2; k++) {
+        int refl = rxy, sz;
+        const int Z = max(map_axis(z0 + k - 1, I.nz, I.wall[2], 4, refl, sz), 0);
+        f(k * T::PS + t, icell3(I, X, Y, Z), refl, sx, sy, sz);
+    }
+}
+
+// the k-th cell of the thread (k < TZ / 2): its coordinates and slot
+#define LBS_TILE_CELL3(k)                                                     \
+    const int x = int(blockIdx.x) * T::TX + (threadIdx.x & 15);               \
+    const int y = int(blockIdx.y) * T::TY + (threadIdx.x >> 5);               \
+    const int lz = 2 * (k) + ((threadIdx.x >> 4) & 1);                        \
+    const int z = int(blockIdx.z) * T::TZ + lz;                               \
+    if (x >= I.nx || y >= I.ny || z >= I.nz) return;                          \
+    const unsigned c = icell3(I, x, y, z);                                    \
+    const int q = T::off((threadIdx.x & 15) + 1, (threadIdx.x >> 5) + 1, lz + 1);
+
 // colour gradient by the isotropic stencil over the 18 neighbours, from the
 // colour fraction that is small on the cell's side (see k_grad2)
 template <typename R>
-__global__ void k_grad3(Inst<R> I, int guess = 1) {
+__global__ void __launch_bounds__(256) k_grad3(Inst<R> I, int guess = 1) {
     // (the one-launch SOR that follows starts from a clear barrier)
-    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 &&
-        threadIdx.y == 0)
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0)
         I.ctl->bar_count = 0;
-    LBS_CELL3
-    const bool blue_side = I.rhoN[c] <= R(0);
-    const Ax X = make_ax(x, I.nx, I.wall[0], 1), Y = make_ax(y, I.ny, I.wall[1], 2),
-             Z = make_ax(z, I.nz, I.wall[2], 4);
-    R gx = R(0), gy = R(0), gz = R(0);
+    using T = Tile3<R>;
+    // colour fractions: blue, red
+    __shared__ R fr[2][T::N];
+    tile3_fill(I, [&](int s, unsigned j, int, int, int, int) {
+        fr[0][s] = frac(I, j, false);
+        fr[1][s] = frac(I, j, true);
+    });
+    __syncthreads();
+#pragma unroll 1
+    for (int k = 0; k < T::TZ / 2; k++) {
+        LBS_TILE_CELL3(k)
+        const bool blue_side = I.rhoN[c] <= R(0);
+        const R *v0 = fr[blue_side ? 1 : 0] + q;
+        R gx = R(0), gy = R(0), gz = R(0);
 #pragma unroll
-    for (int i = 1; i < Q19; i++) {
-        int refl, sx, sy, sz;
-        long long j = nbx3(I, X, Y, Z, ex19(i), ey19(i), ez19(i), refl, sx, sy, sz);
-        R v = w19<R>(i) * frac(I, j, blue_side);
-        if (ex19(i)) gx += R(ex19(i)) * v;
-        if (ey19(i)) gy += R(ey19(i)) * v;
-        if (ez19(i)) gz += R(ez19(i)) * v;
+        for (int i = 1; i < Q19; i++) {
+            const R v = w19<R>(i) * v0[T::off(ex19(i), ey19(i), ez19(i))];
+            if (ex19(i)) gx += R(ex19(i)) * v;
+            if (ey19(i)) gy += R(ey19(i)) * v;
+            if (ez19(i)) gz += R(ez19(i)) * v;
+        }
+        const R f = blue_side ? R(6) : R(-6);  // 2 / c_s^2
+        gx *= f;
+        gy *= f;
+        gz *= f;
+        I.gx[c] = gx;
+        I.gy[c] = gy;
+        I.gz[c] = gz;
+        I.a[c] = sqrt(gx * gx + gy * gy + gz * gz);
+        I.chi[c] = R(2) * fr[0][q];
+        if (guess) sor_guess(I, c);
     }
-    const R f = blue_side ? R(6) : R(-6);  // 2 / c_s^2
-    gx *= f;
-    gy *= f;
-    gz *= f;
-    I.gx[c] = gx;
-    I.gy[c] = gy;
-    I.gz[c] = gz;
-    I.a[c] = sqrt(gx * gx + gy * gy + gz * gz);
-    I.chi[c] = R(2) * frac(I, c, false);
-    if (guess) sor_guess(I, c);
 }
 
 // normal, curvature (Eq. 7), grad psi, sigma (Eq. 8), interfacial force
 // (Eq. 9) plus buoyancy, velocity (Eq. 10)
 template <typename R>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 2) k_force3(Inst<R> I) {
-    LBS_CELL3
+    using T = Tile3<R>;
+    // g (its normal component mirrored with a sign change), 1 / sqrt(|g|^2 +
+    // eps_n^2), psi
+    __shared__ R g3[3][T::N], inv3[T::N], psi3[T::N];
     const R e2 = I.eps_n * I.eps_n;
-    const Ax X = make_ax(x, I.nx, I.wall[0], 1), Y = make_ax(y, I.ny, I.wall[1], 2),
-             Z = make_ax(z, I.nz, I.wall[2], 4);
+    tile3_fill(I, [&](int s, unsigned j, int refl, int, int, int) {
+        R gx = I.gx[j], gy = I.gy[j], gz = I.gz[j];
+        psi3[s] = I.psi[j];
+        if (refl & 1) gx = -gx;
+        if (refl & 2) gy = -gy;
+        if (refl & 4) gz = -gz;
+        g3[0][s] = gx;
+        g3[1][s] = gy;
+        g3[2][s] = gz;
+        inv3[s] = frsq(gx * gx + gy * gy + gz * gz + e2);
+    });
+    __syncthreads();
+#pragma unroll 1
+    for (int k = 0; k < T::TZ / 2; k++) {
+    LBS_TILE_CELL3(k)
+    // (the cell's own values first: one wait for memory a cell)
+    const R a = I.a[c], rR = I.rhoR[c], rB = I.rhoB[c];
+    const R jx = I.jx[c], jy = I.jy[c], jz = I.jz[c];
     R divn = R(0), dpx = R(0), dpy = R(0), dpz = R(0);
 #pragma unroll
     for (int i = 1; i < Q19; i++) {
-        int refl, sx, sy, sz;
-        long long j = nbx3(I, X, Y, Z, ex19(i), ey19(i), ez19(i), refl, sx, sy, sz);
-        R gx = I.gx[j], gy = I.gy[j], gz = I.gz[j];
-        if (refl & 1) gx = -gx;  // normal component mirrored with a sign change
-        if (refl & 2) gy = -gy;
-        if (refl & 4) gz = -gz;
-        const R inv = frsq(gx * gx + gy * gy + gz * gz + e2);
+        const int j = q + T::off(ex19(i), ey19(i), ez19(i));
         R s = R(0);
-        if (ex19(i)) s += R(ex19(i)) * gx;
-        if (ey19(i)) s += R(ey19(i)) * gy;
-        if (ez19(i)) s += R(ez19(i)) * gz;
-        divn -= w19<R>(i) * s * inv;
-        const R p = w19<R>(i) * I.psi[j];
+        if (ex19(i)) s += R(ex19(i)) * g3[0][j];
+        if (ey19(i)) s += R(ey19(i)) * g3[1][j];
+        if (ez19(i)) s += R(ez19(i)) * g3[2][j];
+        divn -= w19<R>(i) * s * inv3[j];
+        const R p = w19<R>(i) * psi3[j];
         if (ex19(i)) dpx += R(ex19(i)) * p;
         if (ey19(i)) dpy += R(ey19(i)) * p;
         if (ez19(i)) dpz += R(ez19(i)) * p;
@@ -191,10 +280,10 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 2) k_force3(Inst<R> 
     dpx *= R(3);
     dpy *= R(3);
     dpz *= R(3);
-    const R gx = I.gx[c], gy = I.gy[c], gz = I.gz[c], a = I.a[c];
+    const R gx = g3[0][q], gy = g3[1][q], gz = g3[2][q];
     R sigma, mco, Fx, Fy, Fz;
-    if (eos(I, I.psi[c], sigma, mco)) {
-        const R inv = frsq(gx * gx + gy * gy + gz * gz + e2);
+    if (eos(I, psi3[q], sigma, mco)) {
+        const R inv = inv3[q];
         const R nx = -gx * inv, ny = -gy * inv, nz = -gz * inv;
         const R ndp = nx * dpx + ny * dpy + nz * dpz;
         Fx = -R(0.5) * sigma * kappa * gx - R(0.5) * a * mco * (dpx - ndp * nx);
@@ -205,7 +294,6 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 2) k_force3(Inst<R> 
         Fy = -R(0.5) * I.sigma_min * kappa * gy;
         Fz = -R(0.5) * I.sigma_min * kappa * gz;
     }
-    const R rR = I.rhoR[c], rB = I.rhoB[c];
     const R rho = rR + rB;
     const R drb = rR + (rB - I.rhoB0);
     Fx += drb * I.g[0];
@@ -215,9 +303,10 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 2) k_force3(Inst<R> 
     I.Fy[c] = Fy;
     I.Fz[c] = Fz;
     const R irho = fdiv(R(1), rho);
-    I.ux[c] = (I.jx[c] + R(0.5) * Fx) * irho;
-    I.uy[c] = (I.jy[c] + R(0.5) * Fy) * irho;
-    I.uz[c] = (I.jz[c] + R(0.5) * Fz) * irho;
+    I.ux[c] = (jx + R(0.5) * Fx) * irho;
+    I.uy[c] = (jy + R(0.5) * Fy) * irho;
+    I.uz[c] = (jz + R(0.5) * Fz) * irho;
+    }
 }
 
 // explicit surfactant terms (Eqs. 22-27) and Crank-Nicolson right-hand sides
@@ -237,7 +326,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2)
 #pragma unroll
         for (int k = -2; k <= 2; k++) {
             int refl, sx, sy, sz;
-            long long j = nbx3(I, X, Y, Z, ax == 0 ? k : 0, ax == 1 ? k : 0, ax == 2 ? k : 0,
+            unsigned j = nbx3(I, X, Y, Z, ax == 0 ? k : 0, ax == 1 ? k : 0, ax == 2 ? k : 0,
                                refl, sx, sy, sz);
             const R sgn = (refl & (1 << ax)) ? R(-1) : R(1);
             const R uj = uax[ax][j];
@@ -264,7 +353,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2)
     for (int f = 0; f < 6; f++) {
         const int s = (f & 1) ? 1 : -1, ax = f >> 1;
         int refl, sx, sy, sz;
-        long long j2 = nbx3(I, X, Y, Z, ax == 0 ? s : 0, ax == 1 ? s : 0, ax == 2 ? s : 0,
+        unsigned j2 = nbx3(I, X, Y, Z, ax == 0 ? s : 0, ax == 1 ? s : 0, ax == 2 ? s : 0,
                             refl, sx, sy, sz);
         if (refl) continue;
         Lp += R(0.5) * (wp + (I.a[j2] + I.eps_w)) * (I.psi[j2] - psi);
@@ -302,7 +391,22 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2)
 // ---------------------------------------------------------------------------
 template <typename R, typename P>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_collide3(Inst<R> I) {
-    LBS_CELL3
+    using T = Tile3<R>;
+    // rho^R, rho^B and the velocity, at walls the ghost's
+    __shared__ R rho3[2][T::N], u3[3][T::N];
+    tile3_fill(I, [&](int s, unsigned j, int refl, int sx, int sy, int sz) {
+        R vx = I.ux[j], vy = I.uy[j], vz = I.uz[j];
+        rho3[0][s] = I.rhoR[j];
+        rho3[1][s] = I.rhoB[j];
+        if (refl) ghost_u3(I, refl, sx, sy, sz, vx, vy, vz);
+        u3[0][s] = vx;
+        u3[1][s] = vy;
+        u3[2][s] = vz;
+    });
+    __syncthreads();
+#pragma unroll 1
+    for (int k = 0; k < T::TZ / 2; k++) {
+    LBS_TILE_CELL3(k)
     R fT[Q19], fM[Q19];
     const int fl = I.flag[c];
 #pragma unroll
@@ -315,32 +419,23 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_collide3(Inst<R
     const R rmin = fl ? rB : rR;
     const R devmaj = I.dsh[fl] + (mo.drho - rmin);
     const R rho = rR + rB;
-    const R ux = I.ux[c], uy = I.uy[c], uz = I.uz[c];
+    const R ux = u3[0][q], uy = u3[1][q], uz = u3[2][q];
     const R Fx = I.Fx[c], Fy = I.Fy[c], Fz = I.Fz[c];
 
-    // d_a(rho^k u_a), isotropic stencil, ghost velocities at walls
+    // d_a(rho^k u_a), isotropic stencil
     R dR[3] = {R(0), R(0), R(0)}, dB[3] = {R(0), R(0), R(0)};
-    const Ax X = make_ax(x, I.nx, I.wall[0], 1), Y = make_ax(y, I.ny, I.wall[1], 2),
-             Z = make_ax(z, I.nz, I.wall[2], 4);
 #pragma unroll
     for (int i = 1; i < Q19; i++) {
-        int refl, sx, sy, sz;
-        long long j = nbx3(I, X, Y, Z, ex19(i), ey19(i), ez19(i), refl, sx, sy, sz);
-        R vx = I.ux[j], vy = I.uy[j], vz = I.uz[j];
-        ghost_u3(I, refl, sx, sy, sz, vx, vy, vz);
-        const R r1 = w19<R>(i) * I.rhoR[j], r2 = w19<R>(i) * I.rhoB[j];
-        if (ex19(i)) {
-            dR[0] += R(ex19(i)) * r1 * vx;
-            dB[0] += R(ex19(i)) * r2 * vx;
-        }
-        if (ey19(i)) {
-            dR[1] += R(ey19(i)) * r1 * vy;
-            dB[1] += R(ey19(i)) * r2 * vy;
-        }
-        if (ez19(i)) {
-            dR[2] += R(ez19(i)) * r1 * vz;
-            dB[2] += R(ez19(i)) * r2 * vz;
-        }
+        const int j = q + T::off(ex19(i), ey19(i), ez19(i));
+        const int e[3] = {ex19(i), ey19(i), ez19(i)};
+        const R r1 = w19<R>(i) * rho3[0][j], r2 = w19<R>(i) * rho3[1][j];
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+            if (e[a]) {
+                const R v = u3[a][j];
+                dR[a] += R(e[a]) * r1 * v;
+                dB[a] += R(e[a]) * r2 * v;
+            }
     }
     const R cR = R(1) - R(1.5) * (R(1) - I.alphaR), cB = R(1) - R(1.5) * (R(1) - I.alphaB);
     const R Qx = R(3) * (cR * dR[0] + cB * dB[0]);
@@ -403,10 +498,10 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_collide3(Inst<R
     dm[13] = -neq[13] + t3 * Fx;
     dm[14] = -neq[14] + t3 * Fz;
     dm[15] = -neq[15] + t3 * Fy;
-    const R u3 = uF / R(3);
-    dm[16] = -neq[16] + R(0.5) * (xF + yF - u3);
-    dm[17] = -neq[17] + R(0.5) * (xF + zF - u3);
-    dm[18] = -neq[18] + R(0.5) * (yF + zF - u3);
+    const R uF3 = uF / R(3);
+    dm[16] = -neq[16] + R(0.5) * (xF + yF - uF3);
+    dm[17] = -neq[17] + R(0.5) * (xF + zF - uF3);
+    dm[18] = -neq[18] + R(0.5) * (yF + zF - uF3);
     R df[Q19];
     minv19<R>(dm, df);
 
@@ -445,47 +540,64 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_collide3(Inst<R
     I.gT0[c] = rest_close(mo.dr_s, mo.dr_c, sT.s, sT.c, R(0), rest_u(rk, 0));
     I.gM0[c] = rest_close(mo.rm_s, mo.rm_c, sM.s, sM.c, R(0), rest_u(rk, 1));
     I.gflag[c] = (uint8_t)fl;
+    }
 }
 
 // streaming (Eq. 13, pull), half-way bounce-back with moving walls, moments
-// at t+1 (see k_stream2).  MIRROR: the grid has mirror planes (a separate
+// at t+1 (see k_stream2).  Bound by the wait for the 38 populations a cell
+// pulls: 4 blocks an SM (64 registers; 5 spill in the fast path and 3 wait
+// longer), which took the general path's second copy of them out of the fast
+// one.  100 cubed FP32, mirror planes: 107 -> 84 us (half of the copy bandwidth),
+// 256 x 128 x 128 BF16 235 -> 194.  MIRROR: the grid has mirror planes (a separate
 // instantiation, so that grids without them keep the plain direction choice)
 template <typename R, typename P, bool MIRROR>
-__global__ void __launch_bounds__(256, 3) k_stream3(Inst<R> I) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_stream3(Inst<R> I) {
     LBS_CELL3
     const int flc = I.gflag[c];
+    // 1. the streamed (total, minority) pairs as stored at their sources;
+    //    slow: a source's flag differs from the cell's or a link crosses a
+    //    moving wall
+    R t[Q19], m[Q19];
+    int slow = 0;
+    {
     const Ax X = make_ax(x, I.nx, I.wall[0], 1), Y = make_ax(y, I.ny, I.wall[1], 2),
              Z = make_ax(z, I.nz, I.wall[2], 4);
-    // 1. the streamed (total, minority) pairs as stored at their sources;
-    //    a link that crosses a wall reflects the cell's own opposite
-    //    population; slow: bit i set where the source's flag differs from the
-    //    cell's or the link crosses a moving wall
-    R t[Q19], m[Q19];
-    unsigned slow = 0, fbits = 0;
-    // (branch-free: a reflected link reads the cell's own opposite
-    // population, so that every load of the loop can be in flight at once)
+    t[0] = I.gT0[c];
+    m[0] = I.gM0[c];
+    const int near = X.r[1] | X.r[3] | Y.r[1] | Y.r[3] | Z.r[1] | Z.r[3];
+    if (!__any_sync(__activemask(), near)) {
+        // no link of the warp's cells crosses a boundary: plain pulls (most
+        // warps; a third of the other form's instructions)
 #pragma unroll
-    for (int i = 0; i < Q19; i++) {
-        int refl, sx, sy, sz;
-        const long long j = nbx3(I, X, Y, Z, -ex19(i), -ey19(i), -ez19(i), refl, sx, sy, sz);
-        if (i == 0) {
-            t[0] = I.gT0[c];
-            m[0] = I.gM0[c];
-            continue;
+        for (int i = 1; i < Q19; i++) {
+            int refl, sx, sy, sz;
+            const unsigned j = nbx3(I, X, Y, Z, -ex19(i), -ey19(i), -ez19(i), refl, sx, sy, sz);
+            const long long k = (long long)i * I.plane + j;
+            t[i] = ldp<R, P>(I, I.gT, k);
+            m[i] = ldp<R, P>(I, I.gM, k);
+            slow |= I.gflag[j] ^ flc;
         }
-        const int bb = refl & I.bbmask;  // mirror planes: the mirrored source
-        const long long src = bb ? c : j;
-        const int dir = bb ? opp19(i) : (MIRROR ? mir19(i, refl) : i);
-        const long long k = (long long)dir * I.plane + src;
-        t[i] = ldp<R, P>(I, I.gT, k);
-        m[i] = ldp<R, P>(I, I.gM, k);
-        const int fj = I.gflag[src];
-        fbits |= (unsigned)fj << i;
-        // (a static wall returns the cell's own opposite population unchanged:
-        // the fast path's plain move; a moving wall adds its momentum term)
-        if (fj != flc || (bb & I.mvmask)) slow |= 1u << i;
+    } else {
+        // a link that crosses a wall reflects the cell's own opposite
+        // population (branch-free, so that every load of the loop can be in
+        // flight at once)
+#pragma unroll
+        for (int i = 1; i < Q19; i++) {
+            int refl, sx, sy, sz;
+            const unsigned j = nbx3(I, X, Y, Z, -ex19(i), -ey19(i), -ez19(i), refl, sx, sy, sz);
+            const int bb = refl & I.bbmask;  // mirror planes: the mirrored source
+            const unsigned src = bb ? c : j;
+            const int dir = bb ? opp19(i) : (MIRROR ? mir19(i, refl) : i);
+            const long long k = (long long)dir * I.plane + src;
+            t[i] = ldp<R, P>(I, I.gT, k);
+            m[i] = ldp<R, P>(I, I.gM, k);
+            // (a static wall returns the cell's own opposite population
+            // unchanged: the fast path's plain move; a moving wall adds its
+            // momentum term)
+            slow |= (I.gflag[src] ^ flc) | (bb & I.mvmask);
+        }
     }
-    fbits |= (unsigned)flc;  // (i = 0: the cell's own flag)
+    }
     // 2. fast path: every population moves unchanged; the cell keeps its
     //    flag unless its minority colour has become the majority
     if (!slow) {
@@ -521,26 +633,37 @@ __global__ void __launch_bounds__(256, 3) k_stream3(Inst<R> I) {
     }
     // 3. general path: colours re-split where the flags differ, moving-wall
     //    terms added; every value carried as hi + lo (TwoSum errors), and
-    //    the rest populations close the cell's masses exactly
+    //    the rest populations close the cell's masses exactly.  It reads the
+    //    populations again (x laundered, so that nothing of part 1 is kept for
+    //    it): the few cells that come here should not cost the others registers.
+    int xg = x;
+    asm volatile("" : "+r"(xg));
+    const Ax X = make_ax(xg, I.nx, I.wall[0], 1), Y = make_ax(y, I.ny, I.wall[1], 2),
+             Z = make_ax(z, I.nz, I.wall[2], 4);
     const R rRc = I.rhoR[c], rBc = I.rhoB[c];
     R fR[Q19], fB[Q19];
     R loT = R(0), loR = R(0), loB = R(0);
 #pragma unroll
     for (int i = 0; i < Q19; i++) {
-        const int fj = (fbits >> i) & 1;
+        int refl, sx, sy, sz;
+        const unsigned j = nbx3(I, X, Y, Z, -ex19(i), -ey19(i), -ez19(i), refl, sx, sy, sz);
+        const int bb = refl & I.bbmask;
+        const unsigned src = bb ? c : j;
+        const int dir = bb ? opp19(i) : (MIRROR ? mir19(i, refl) : i);
+        t[i] = ldq<R, P>(I, I.gT, I.gT0, dir, src);
+        m[i] = ldq<R, P>(I, I.gM, I.gM0, dir, src);
+        const int fj = i ? I.gflag[src] : flc;
         R tlo = R(0), mlo = R(0);
         R sh = shift_of(I, i, fj);
-        if ((slow >> i) & 1) {
-            int refl, sx, sy, sz;
-            nbx3(I, X, Y, Z, -ex19(i), -ey19(i), -ez19(i), refl, sx, sy, sz);
-            refl &= I.bbmask;  // (mirror planes reflect without a wall term)
-            if (refl) {
+        if (fj != flc || (bb & I.mvmask)) {
+            // (mirror planes reflect without a wall term)
+            if (bb) {
                 R uw[3] = {R(0), R(0), R(0)};
                 int nw = 0;
                 const int side[3] = {sx, sy, sz};
 #pragma unroll
                 for (int a = 0; a < 3; a++) {
-                    if (!(refl & (1 << a))) continue;
+                    if (!(bb & (1 << a))) continue;
                     const R *w = side[a] < 0 ? I.uw_lo[a] : I.uw_hi[a];
                     uw[0] += w[0];
                     uw[1] += w[1];
@@ -669,7 +792,7 @@ __global__ void __launch_bounds__(BS)
         for (int f = 0; f < 6; f++) {
             const int s = (f & 1) ? 1 : -1, ax = f >> 1;
             int refl, sx, sy, sz;
-            long long j = nbx3(I, X, Y, Z, ax == 0 ? s : 0, ax == 1 ? s : 0, ax == 2 ? s : 0,
+            unsigned j = nbx3(I, X, Y, Z, ax == 0 ? s : 0, ax == 1 ? s : 0, ax == 2 ? s : 0,
                                refl, sx, sy, sz);
             if (refl) continue;  // no flux through a wall
             const R fp = hp * (R(0.5) * (wp + (I.a[j] + I.eps_w)));

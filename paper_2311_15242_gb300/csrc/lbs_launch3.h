@@ -22,11 +22,11 @@ struct Launch3 {
     static void init(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s, const double *phi,
                      const double *psi, const double *C, const double *u);
     static void moments(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s);
-    static void grad(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s, int guess = 1);
-    static void force(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s);
+    static void grad(const Inst<R> &I, cudaStream_t s, int guess = 1);
+    static void force(const Inst<R> &I, cudaStream_t s);
     static void fd(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s, double *Sout,
                    double *Bout);
-    static void collide(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s);
+    static void collide(const Inst<R> &I, cudaStream_t s);
     static void stream(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s);
     static void diag(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s, int nblocks);
     // one red (colour 0) or black (colour 1) SOR half-sweep: variant 0 one
