@@ -2,11 +2,13 @@
 // the coupled step: different grids, Eotvos and Biot numbers, confinement)
 // advanced together.
 //
-// Every phase of the step is one launch for the whole batch: a grid of
-// (SM count x resident blocks) blocks walks a work list of (instance, tile)
-// items, copies the instance's descriptor into shared memory when the
-// instance changes and runs the same per-cell bodies as the single-instance
-// kernels.  The SOR rounds of all instances share one WHILE node: each
+// In FP32 arithmetic everything up to the moments of t+1 is the fused step, one
+// launch an instance, side by side (kb_fused2).  Every other phase is one launch
+// for the whole batch: a grid of (SM count x resident blocks) blocks walks a
+// work list of (instance, tile) items, copies the instance's descriptor into
+// shared memory when the instance changes and runs the same per-cell bodies as
+// the single-instance kernels; FP64, bound by its arithmetic, of which a tile's
+// halo would be a quarter more, takes all phases that way.  The SOR rounds of all instances share one WHILE node: each
 // instance keeps its own round counter, convergence test and ping-pong
 // parity, a converged instance's tiles skip the remaining rounds, and the
 // loop ends when no instance is still iterating.  In FP32 arithmetic, where
@@ -24,8 +26,8 @@
 #include <new>
 #include <vector>
 
+#include "lbs_fused2.cuh"
 #include "lbs_internal.h"
-#include "lbs_k2d.cuh"
 #include "lbs_solve2.cuh"
 
 using namespace lbs;
@@ -41,8 +43,7 @@ struct BatchCtl {
     int active;           // instances still iterating in the current solve
 };
 
-// OP_FDCOLLIDE_G: also leaves the solve's starting guess in psi2, C2 (kb_solve2)
-enum { OP_FORCE, OP_FDCOLLIDE, OP_STREAM, OP_GRAD, OP_SCALE, OP_FDCOLLIDE_G, NOPS };
+enum { OP_FORCE, OP_FDCOLLIDE, OP_STREAM, OP_GRAD, OP_SCALE, NOPS };
 
 // copy descriptor k into shared memory (all threads; uniform) and return
 // whether the instance is alive (an instance whose total went non-finite is
@@ -78,32 +79,38 @@ __global__ void kb_cells2(const Inst<R> *__restrict__ insts, const WorkItem *__r
         const int x = it.x0 + threadIdx.x, y = it.y0 + threadIdx.y;
         if (OP == OP_FORCE)
             force2_cell(sI, x, y);
-        else if (OP == OP_FDCOLLIDE || OP == OP_FDCOLLIDE_G) {
+        else if (OP == OP_FDCOLLIDE) {
             // (the explicit surfactant terms and the collision in one pass)
             fd2_cell(sI, x, y, nullptr, nullptr);
-            if (OP == OP_FDCOLLIDE_G && x < sI.nx && y < sI.ny) {
-                // (2 x^n - x^(n-1), see sor_guess; neighbours read psi, C, so
-                // the guess goes to the second buffers)
-                const long long c = (long long)y * sI.pitch + x;
-                const R p = sI.psi[c], q = sI.C[c];
-                sI.psi2[c] = R(2) * p - sI.psip[c];
-                sI.C2[c] = R(2) * q - sI.Cp[c];
-                sI.psip[c] = p;
-                sI.Cp[c] = q;
-            }
             collide2_cell<R, P>(sI, x, y);
         }
-        else if (OP == OP_STREAM) {
-            // (kb_solve2's barrier of this instance starts from a clear count)
-            if (it.x0 == 0 && it.y0 == 0 && threadIdx.x == 0 && threadIdx.y == 0)
-                sI.ctl->bar_count = 0;
+        else if (OP == OP_STREAM)
             stream2_cell<R, P>(sI, x, y);
+        else if (OP == OP_GRAD) {
+            // (after the fused step the moments of t+1 are in the next set and
+            // the starting guess is made)
+            if (!sI.pop_pp)
+                grad2_cell(sI, x, y);
+            else if (x < sI.nx && y < sI.ny)
+                grad2_next_cell(sI, mom_of_step(sI, sI.ctl->step + 1), x, y);
         }
-        else if (OP == OP_GRAD)
-            grad2_cell(sI, x, y);
         else
             scale2_cell(sI, x, y, 0);
     }
+}
+
+// the fused step (k_lbfd2) of one instance; the batch's instances run side by
+// side on streams of their own between two events (branches of the graph).  One
+// launch over all instances with the descriptors in memory took 170 us for 8 of
+// them (0.85 M cells, FP16), no less than the three phases it replaced (force,
+// surfactant terms and collision, streaming): every field of a descriptor came
+// through shared memory and 65 registers were spilled; as launch parameters
+// they are operands of the arithmetic and the 8 take about 130 us (a step 306 ->
+// 268 us; 64 instances, 7.1 M cells, 240 steps and their fields 577 -> 501 ms).
+template <typename R, typename P, int TX, int TY>
+__global__ void __launch_bounds__(TX *TY, 1024 / (TX * TY)) kb_fused2(Inst<R> I) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    lbfd2_block<R, P, TX, TY, true>(I, blockIdx.x * TX, blockIdx.y * TY, smem_raw);
 }
 
 // opens the SOR solve of every live instance in the work lists (act[k])
@@ -300,6 +307,14 @@ struct Batch : lbs_batch {
     std::vector<int> act;      // host flags: instance in the work lists
     std::vector<int> st;       // sticky per-instance status (lbs_status codes)
     WorkItem *d_cells = nullptr, *d_sor = nullptr, *d_surf = nullptr;
+    // kb_fused2: its tile (16 x 8 or 32 x 16), the instances' descriptors, and
+    // the streams of the launches beside the batch's own
+    static constexpr bool kFused = sizeof(R) == 4;
+    static constexpr int kSide = 7;
+    bool fused_small = false;
+    std::vector<Inst<R>> insts;
+    cudaStream_t side[kSide] = {};
+    cudaEvent_t fork = nullptr, joined[kSide] = {};
     // kb_solve2: its form (K sweeps a round, NR rounds between barriers), work
     // and waves; gang.fn == nullptr: one launch a round instead
     struct {
@@ -333,6 +348,11 @@ struct Batch : lbs_batch {
         cudaFree(d_sor);
         cudaFree(d_surf);
         cudaFree(d_gang);
+        for (int i = 0; i < kSide; i++) {
+            if (side[i]) cudaStreamDestroy(side[i]);
+            if (joined[i]) cudaEventDestroy(joined[i]);
+        }
+        if (fork) cudaEventDestroy(fork);
         if (own_ws && ws) cudaFree(ws);
         if (own_stream && stream) cudaStreamDestroy(stream);
     }
@@ -371,7 +391,8 @@ struct Batch : lbs_batch {
             BCK(cudaMalloc(&ws, total));
             own_ws = true;
         }
-        std::vector<Inst<R>> h(n);
+        std::vector<Inst<R>> &h = insts;
+        h.resize(n);
         for (int k = 0; k < n; k++) {
             lbs_ctx *c = new (std::nothrow) lbs_ctx();
             if (!c) return LBS_ENOMEM;
@@ -388,10 +409,10 @@ struct Batch : lbs_batch {
                 berr(this, "internal: descriptor size mismatch");
                 return LBS_EINVAL;
             }
-            // the batch runs the separate per-cell kernels: populations and
-            // moments return to set 0 every step and the SOR starting guess
-            // sits in psi, C
-            c->impl->set_batch_member();
+            // FP64 runs the separate per-cell kernels: populations and moments
+            // return to set 0 every step and the SOR starting guess sits in
+            // psi, C; the fused step keeps them as a solver of its own does
+            if (!kFused) c->impl->set_batch_member();
             std::memcpy(&h[k], c->impl->inst(), sizeof(Inst<R>));
             if (p[k].sor_max_iter > max_iter) max_iter = p[k].sor_max_iter;
         }
@@ -409,7 +430,67 @@ struct Batch : lbs_batch {
             BCK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)sor_smem<R>(v)));
         }
+        if constexpr (kFused) {
+            BCK(cudaFuncSetAttribute((void *)kb_fused2<R, P, 32, 16>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)Fuse2<R, 32, 16>::bytes()));
+            BCK(cudaFuncSetAttribute((void *)kb_fused2<R, P, 16, 8>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)Fuse2<R, 16, 8>::bytes()));
+            BCK(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
+            for (int i = 0; i < std::min(n - 1, (int)kSide); i++) {
+                BCK(cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking));
+                BCK(cudaEventCreateWithFlags(&joined[i], cudaEventDisableTiming));
+            }
+        }
         return set_tiles(32, 8, 0);
+    }
+
+    template <int TX, int TY>
+    long long fused_tiles() const {
+        long long t = 0;
+        for (int k = 0; k < n; k++)
+            if (act[k])
+                t += (long long)((insts[k].nx + TX - 1) / TX) * ((insts[k].ny + TY - 1) / TY);
+        return t;
+    }
+    // the fused step's tile: the smaller ones as for a solver of its own, where
+    // the larger would leave half of the SMs idle
+    void set_fused() {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        fused_small = fused_tiles<32, 16>() <= sms / 2;
+    }
+    template <int TX, int TY>
+    void launch_fused(int k, cudaStream_t s) {
+        const Inst<R> &I = insts[k];
+        kb_fused2<R, P, TX, TY><<<dim3((I.nx + TX - 1) / TX, (I.ny + TY - 1) / TY), TX * TY,
+                                  Fuse2<R, TX, TY>::bytes(), s>>>(I);
+    }
+    // the fused step of every active instance on s and the streams beside it
+    int enqueue_fused(cudaStream_t s) {
+        int live = 0;
+        for (int k = 0; k < n; k++) live += act[k];
+        const int ns = std::min(live - 1, (int)kSide);  // streams beside s
+        if (ns > 0) {
+            BCK(cudaEventRecord(fork, s));
+            for (int i = 0; i < ns; i++) BCK(cudaStreamWaitEvent(side[i], fork, 0));
+        }
+        for (int k = 0, at = 0; k < n; k++) {
+            if (!act[k]) continue;
+            const int i = at++ % (ns + 1);
+            cudaStream_t t = i ? side[i - 1] : s;
+            if (fused_small)
+                launch_fused<16, 8>(k, t);
+            else
+                launch_fused<32, 16>(k, t);
+        }
+        for (int i = 0; i < ns; i++) {
+            BCK(cudaEventRecord(joined[i], side[i]));
+            BCK(cudaStreamWaitEvent(s, joined[i], 0));
+        }
+        return LBS_OK;
     }
 
     // resident blocks of kernel f x SM count (a persistent grid), capped by the work
@@ -549,10 +630,17 @@ struct Batch : lbs_batch {
         n_surf = (int)surf.size();
         BCK(cudaMemcpy(d_act, act.data(), n * sizeof(int), cudaMemcpyHostToDevice));
         const int th = tx * ty;
-        const void *fk[NOPS] = {(void *)kb_cells2<R, P, OP_FORCE>, (void *)kb_cells2<R, P, OP_FDCOLLIDE>,
-                             (void *)kb_cells2<R, P, OP_STREAM>, (void *)kb_cells2<R, P, OP_GRAD>,
-                             (void *)kb_cells2<R, P, OP_SCALE>, (void *)kb_cells2<R, P, OP_FDCOLLIDE_G>};
-        for (int o = 0; o < NOPS; o++) g_cells[o] = persistent_grid(fk[o], th, 0, n_cells);
+        const void *fk[NOPS] = {nullptr, nullptr, nullptr, (void *)kb_cells2<R, P, OP_GRAD>,
+                                (void *)kb_cells2<R, P, OP_SCALE>};
+        if constexpr (!kFused) {
+            fk[OP_FORCE] = (void *)kb_cells2<R, P, OP_FORCE>;
+            fk[OP_FDCOLLIDE] = (void *)kb_cells2<R, P, OP_FDCOLLIDE>;
+            fk[OP_STREAM] = (void *)kb_cells2<R, P, OP_STREAM>;
+        } else {
+            set_fused();
+        }
+        for (int o = 0; o < NOPS; o++)
+            if (fk[o]) g_cells[o] = persistent_grid(fk[o], th, 0, n_cells);
         g_sor = persistent_grid(sor_kernel(sizeof(R) == 8, sv), sor_vbs(sv), sor_smem<R>(sv), n_sor);
         g_surf = persistent_grid((void *)kb_surf2<R, kSurfBS>, kSurfBS, 0, n_surf);
         return set_gang();
@@ -572,14 +660,15 @@ struct Batch : lbs_batch {
     // the launches of one step of the whole batch
     int enqueue_step(cudaStream_t s, bool capturing) {
         const dim3 blk(tx, ty, 1);
-        kb_cells2<R, P, OP_FORCE><<<g_cells[OP_FORCE], blk, 0, s>>>(d_insts, d_cells, n_cells);
-        if (gang.fn)
-            kb_cells2<R, P, OP_FDCOLLIDE_G><<<g_cells[OP_FDCOLLIDE_G], blk, 0, s>>>(
-                d_insts, d_cells, n_cells);
-        else
+        if constexpr (kFused) {
+            int r = enqueue_fused(s);
+            if (r) return r;
+        } else {
+            kb_cells2<R, P, OP_FORCE><<<g_cells[OP_FORCE], blk, 0, s>>>(d_insts, d_cells, n_cells);
             kb_cells2<R, P, OP_FDCOLLIDE><<<g_cells[OP_FDCOLLIDE], blk, 0, s>>>(d_insts, d_cells,
                                                                               n_cells);
-        kb_cells2<R, P, OP_STREAM><<<g_cells[OP_STREAM], blk, 0, s>>>(d_insts, d_cells, n_cells);
+            kb_cells2<R, P, OP_STREAM><<<g_cells[OP_STREAM], blk, 0, s>>>(d_insts, d_cells, n_cells);
+        }
         if (gang.fn) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(gang.blocks, 1, 1);
@@ -772,10 +861,14 @@ struct Batch : lbs_batch {
         return LBS_OK;
     }
 
-    // launches of one step: 3 cell phases (fd fused with collide) and kb_solve2;
-    // or 4 cell phases, the SOR opener, the rounds of the slowest instance at the last diagnostics, the
-    // total and the rescale
-    int kernel_count() const override { return gang.fn ? 4 : 7 + last_rounds; }
+    // launches of one step: the fused steps and kb_solve2; or the fused steps
+    // (FP64: 3 cell phases), the gradient, the SOR opener, the rounds of the slowest
+    // instance at the last diagnostics, the total and the rescale
+    int kernel_count() const override {
+        int live = 0;
+        for (int k = 0; k < n; k++) live += act[k];
+        return (kFused ? live : 3) + (gang.fn ? 1 : 4 + last_rounds);
+    }
 
     int set_graph(int on) override {
         use_graph = bool(on);

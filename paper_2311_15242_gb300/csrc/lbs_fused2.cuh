@@ -101,7 +101,8 @@ __device__ __forceinline__ PopSets<R> pop_sets(const Inst<R> &I) {
 // out, and a differently compiled copy could fuse other multiply-adds.
 template <typename R, typename P, int TX, int TY>
 __device__ __forceinline__ void lbfd2_tile(const Inst<R> &I, const PopSets<R> &ps,
-                                           unsigned char *smem_raw, const bool EDGE) {
+                                           const int x0, const int y0, unsigned char *smem_raw,
+                                           const bool EDGE) {
     using F = Fuse2<R, TX, TY>;
     constexpr int W3 = F::W3, N3 = F::N3, W2 = F::W2, N2 = F::N2, W1 = F::W1, N1 = F::N1;
     constexpr int NT = F::NT;
@@ -113,7 +114,6 @@ __device__ __forceinline__ void lbfd2_tile(const Inst<R> &I, const PopSets<R> &p
     uint8_t *code3 = (uint8_t *)(pM01 + N1), *flag1 = code3 + N3;
     int16_t *src1 = (int16_t *)(((uintptr_t)(flag1 + N1) + 1) & ~(uintptr_t)1);
     const int tid = threadIdx.x;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
 
     // 2. interface normals n = -g / sqrt(|g|^2 + eps_n^2) (reading R3)
     const R e2 = I.eps_n * I.eps_n;
@@ -583,23 +583,25 @@ __device__ __forceinline__ void lbfd2_tile(const Inst<R> &I, const PopSets<R> &p
     ps.dm.jy[c] = mo.jy;
 }
 
-template <typename R, typename P, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY, (sizeof(R) == 4 ? 1024 : 512) / (TX * TY)) k_lbfd2(Inst<R> I) {
+// the whole step of the tile at (x0, y0), by a block of TX x TY threads; BATCH:
+// unless the instance is dead
+template <typename R, typename P, int TX, int TY, bool BATCH = false>
+__device__ __forceinline__ void lbfd2_block(const Inst<R> &I, const int x0, const int y0,
+                                            unsigned char *smem_raw) {
     using F = Fuse2<R, TX, TY>;
     constexpr int W3 = F::W3, N3 = F::N3, N2 = F::N2, N1 = F::N1;
     constexpr int NT = F::NT;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     // the halo slots this phase fills (layout as in lbfd2_tile)
     R *gx3 = (R *)smem_raw, *gy3 = gx3 + N3, *ps3 = gy3 + N3;
     R *rR2 = ps3 + 3 * N3, *rB2 = rR2 + N2, *jx2 = rB2 + N2, *jy2 = jx2 + N2, *a2 = jy2 + N2;
     R *ch2 = a2 + N2, *Cs2 = ch2 + N2;
     uint8_t *code3 = (uint8_t *)(rR2 + 11 * N2 + 18 * N1);
     const int tid = threadIdx.x;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const PopSets<R> ps = pop_sets(I);
+    if (BATCH && I.ctl->dead) return;
     // the one-launch SOR follows: its grid barrier starts from a clear count
     // whatever an earlier launch that gave up left behind
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) I.ctl->bar_count = 0;
+    if (x0 == 0 && y0 == 0 && tid == 0) I.ctl->bar_count = 0;
 
     // 1. the halo-3 region: g (normal component mirrored at walls and
     //    mirror planes), psi; the halo-2 part also rho^R, rho^B, j, a, chi, C
@@ -639,7 +641,13 @@ __global__ void __launch_bounds__(TX * TY, (sizeof(R) == 4 ? 1024 : 512) / (TX *
     }
     // (the tile meets a wall or mirror plane: block-uniform)
     const bool edge = __syncthreads_or(near_edge) != 0;
-    lbfd2_tile<R, P, TX, TY>(I, ps, smem_raw, edge);
+    lbfd2_tile<R, P, TX, TY>(I, ps, x0, y0, smem_raw, edge);
+}
+
+template <typename R, typename P, int TX, int TY>
+__global__ void __launch_bounds__(TX * TY, (sizeof(R) == 4 ? 1024 : 512) / (TX * TY)) k_lbfd2(Inst<R> I) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    lbfd2_block<R, P, TX, TY>(I, blockIdx.x * TX, blockIdx.y * TY, smem_raw);
 }
 
 // ---------------------------------------------------------------------------
