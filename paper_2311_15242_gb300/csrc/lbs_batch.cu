@@ -187,6 +187,13 @@ __global__ void kb_surf2(const Inst<R> *__restrict__ insts, const WorkItem *__re
     }
 }
 
+// the status words of all instances
+template <typename R>
+__global__ void kb_status(const Inst<R> *__restrict__ insts, int n, int *out) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) out[k] = insts[k].ctl->status;
+}
+
 // one block's tile of one instance in one wave of kb_solve2 (inst < 0: none)
 struct GangItem {
     int inst, bx, by, blk, nb;
@@ -303,6 +310,7 @@ struct Batch : lbs_batch {
     std::vector<lbs_ctx *> ctxs;
     Inst<R> *d_insts = nullptr;
     BatchCtl *d_bc = nullptr;
+    int *d_status = nullptr;   // status words gathered by kb_status
     int *d_act = nullptr;      // instance in the work lists (device copy of act)
     std::vector<int> act;      // host flags: instance in the work lists
     std::vector<int> st;       // sticky per-instance status (lbs_status codes)
@@ -344,6 +352,7 @@ struct Batch : lbs_batch {
         cudaFree(d_insts);
         cudaFree(d_bc);
         cudaFree(d_act);
+        cudaFree(d_status);
         cudaFree(d_cells);
         cudaFree(d_sor);
         cudaFree(d_surf);
@@ -422,6 +431,7 @@ struct Batch : lbs_batch {
         BCK(cudaMemset(d_bc, 0, sizeof(BatchCtl)));
         act.assign(n, 1);
         st.assign(n, 0);
+        BCK(cudaMalloc(&d_status, n * sizeof(int)));
         BCK(cudaMalloc(&d_act, n * sizeof(int)));
         BCK(cudaMemcpy(d_act, act.data(), n * sizeof(int), cudaMemcpyHostToDevice));
         for (int v = 0; v < kSorVariants; v++) {
@@ -785,10 +795,18 @@ struct Batch : lbs_batch {
     }
 
     // reads (and clears on the device) every instance's status into the
-    // sticky host copy; CUDA failures are returned
+    // sticky host copy; CUDA failures are returned.  One launch gathers the
+    // status words and only an instance with one set is asked itself (asking
+    // each cost a synchronisation and a copy an instance, 40 ms for reading the
+    // fields of 64).
     int collect() {
+        std::vector<int> set(n);
+        kb_status<R><<<(n + 127) / 128, 128, 0, stream>>>(d_insts, n, d_status);
+        BCK(cudaGetLastError());
+        BCK(cudaMemcpyAsync(set.data(), d_status, n * sizeof(int), cudaMemcpyDeviceToHost, stream));
         BCK(cudaStreamSynchronize(stream));
         for (int k = 0; k < n; k++) {
+            if (!set[k]) continue;
             int r = ctxs[k]->impl->sync();
             if (r == LBS_ECUDA) {
                 berr(this, "instance %d: %s", k, ctxs[k]->err);
