@@ -40,6 +40,8 @@ void *sor2_kernel(int v) {
     case 6: return (void *)k_sor_tb2<R, LBS_SORV(6)>;
     case 7: return (void *)k_sor_tb2<R, LBS_SORV(7)>;
     case 8: return (void *)k_sor_tb2<R, LBS_SORV(8)>;
+    case kSorSmall:
+        if constexpr (sizeof(R) == 8) return (void *)k_sor_tb2<R, LBS_SORV(kSorSmall)>;
     default: return (void *)k_sor_tb2<R, LBS_SORV(0)>;
     }
 }
@@ -55,6 +57,8 @@ void *sor2_coop_kernel(int v) {
     case 6: return (void *)k_sorfuse2<R, LBS_SORV(6)>;
     case 7: return (void *)k_sorfuse2<R, LBS_SORV(7)>;
     case 8: return (void *)k_sorfuse2<R, LBS_SORV(8)>;
+    case kSorSmall:
+        if constexpr (sizeof(R) == 8) return (void *)k_sorfuse2<R, LBS_SORV(kSorSmall)>;
     default: return (void *)k_sorfuse2<R, LBS_SORV(0)>;
     }
 }
@@ -69,6 +73,7 @@ size_t sor2_smem(int v) {
     case 6: return SorTile<R, LBS_SORV(6)>::smem_bytes();
     case 7: return SorTile<R, LBS_SORV(7)>::smem_bytes();
     case 8: return SorTile<R, LBS_SORV(8)>::smem_bytes();
+    case kSorSmall: return SorTile<R, LBS_SORV(kSorSmall)>::smem_bytes();
     default: return SorTile<R, LBS_SORV(0)>::smem_bytes();
     }
 }
@@ -161,6 +166,19 @@ FusedTile fused_tile_for(int nx, int ny, int sms) {
     const long long tiles =
         (long long)((nx + big.tx - 1) / big.tx) * ((ny + big.ty - 1) / big.ty);
     return tiles <= (sizeof(R) == 8 ? sms : sms / 2) ? fused_tile<R, P, 16, 8>() : big;
+}
+
+// the tile a SOR variant runs: FP64 takes the small tile for variant 0 up to half
+// as many 32 x 16 tiles as SMs.  A round is bound by the FP64 pipes of the SMs
+// that have a tile (two lanes a cycle each); a smaller tile spends more of its
+// work on the halo, 3 cells swept for one instead of 1.9, on up to four times
+// the SMs.  SOR group, 16 sweeps: 128 x 128 (32 tiles) 184 -> 100 us, 192 x 192
+// (72) 186 -> 129; 250 x 250 (128) 186 -> 205.
+template <typename R>
+int sor_variant_for(int v, int nx, int ny, int sms) {
+    const long long tiles = (long long)((nx + sor_vtx(0) - 1) / sor_vtx(0)) *
+                            ((ny + sor_vty(0) - 1) / sor_vty(0));
+    return v == 0 && sizeof(R) == 8 && tiles <= sms / 2 ? kSorSmall : v;
 }
 
 template <typename R, typename P>
@@ -349,14 +367,13 @@ struct Solver : Base {
         stage = (double *)(ws + L.stage_off);
         block = dim3(BX, BY, 1);
         grid = dim3((p->nx + BX - 1) / BX, (p->ny + BY - 1) / BY, p->nz);
-        set_sor_grid();
         const long long rows = (long long)p->ny * p->nz;
         surf_grid = dim3((p->nx + BX - 1) / BX,
                          (unsigned)((rows + BY * SURF_STRIP - 1) / (BY * SURF_STRIP)), 1);
         surf_blocks = (int)(surf_grid.x * surf_grid.y);
         diag_grid = dim3(grid.x, (p->ny + BY * DIAG_STRIP - 1) / (BY * DIAG_STRIP), p->nz);
         diag_blocks = (int)(diag_grid.x * diag_grid.y * diag_grid.z);
-        for (int v = 0; v < kSorVariants; v++)
+        for (int v = 0; v < kSorVariants + (sizeof(R) == 8); v++)  // (and kSorSmall)
             if (sor2_fits(v)) {
                 cudaFuncSetAttribute(sor2_kernel<R>(v),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -368,6 +385,7 @@ struct Solver : Base {
         if (D == 3)
             cudaFuncSetAttribute(Launch3<R, P>::zm_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)Launch3<R, P>::zm_smem());
+        set_sor_grid();  // (asks for the resident blocks: after the shared memory is allowed)
         if (D == 2) {
             int dev = 0, sms = 1;
             cudaGetDevice(&dev);
@@ -384,11 +402,16 @@ struct Solver : Base {
     // half-sweeps in place, 1 = z-marching full sweeps (ping-pong buffers),
     // 2, 3 = red-black half-sweeps in place by column marching (8 or 4 planes)
     int sv = 0;
+    int s2 = 0;  // 2D: the tile that variant sv runs (sor_variant_for)
     void set_sor_grid() {
         using L3 = Launch3<R, P>;
         if (D == 2) {
-            sor_grid = dim3((I.nx + sor_vtx(sv) - 1) / sor_vtx(sv),
-                            (I.ny + sor_vty(sv) - 1) / sor_vty(sv), 1);
+            int dev = 0, sms = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            s2 = sor_variant_for<R>(sv, I.nx, I.ny, sms);
+            sor_grid = dim3((I.nx + sor_vtx(s2) - 1) / sor_vtx(s2),
+                            (I.ny + sor_vty(s2) - 1) / sor_vty(s2), 1);
         } else if (sv == 1) {
             sor_grid = L3::zm_grid(I.nx, I.ny, I.nz);
         } else {
@@ -420,13 +443,17 @@ struct Solver : Base {
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-            if (sor2_fits(sv))
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sor2_coop_kernel<R>(sv),
-                                                              sor_vbs(sv), sor2_smem<R>(sv));
+            if (sor2_fits(s2))
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sor2_coop_kernel<R>(s2),
+                                                              sor_vbs(s2), sor2_smem<R>(s2));
             const long long tiles = (long long)sor_grid.x * sor_grid.y;
             const long long resident = (long long)per_sm * sms;
             coop_blocks = (int)(tiles < resident ? tiles : resident);
-            coop_ok = coop && coop_blocks > 0;
+            // (FP64 only while every tile has an SM: beyond, a launch a round
+            // spreads them better than blocks that wait for each other; SOR,
+            // gradient and total at 250 x 250, 128 tiles: 186 us in one launch,
+            // 217 in several; 300 x 300, 190: 287 and 278; 400 x 400, 325: 520 and 425)
+            coop_ok = coop && coop_blocks > 0 && (sizeof(R) == 4 || s2 == kSorSmall || tiles <= sms);
             set_solve(coop ? sms : 0);
         }
     }
@@ -512,8 +539,8 @@ struct Solver : Base {
         int maxr = sor_rounds();
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(coop_blocks, 1, 1);
-        cfg.blockDim = dim3(sor_vbs(sv), 1, 1);
-        cfg.dynamicSmemBytes = sor2_smem<R>(sv);
+        cfg.blockDim = dim3(sor_vbs(s2), 1, 1);
+        cfg.dynamicSmemBytes = sor2_smem<R>(s2);
         cfg.stream = s;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeCooperative;
@@ -530,7 +557,7 @@ struct Solver : Base {
             return LBS_OK;
         }
         void *args[] = {(void *)&I, (void *)&maxr, (void *)&polls};
-        CK(cudaLaunchKernelExC(&cfg, sor2_coop_kernel<R>(sv), args));
+        CK(cudaLaunchKernelExC(&cfg, sor2_coop_kernel<R>(s2), args));
         return LBS_OK;
     }
     // variant v's shared memory fits a block on this device
@@ -725,10 +752,10 @@ struct Solver : Base {
             if (D == 2) {
                 void *args[] = {(void *)&I, (void *)&h, (void *)&maxr, (void *)&eager};
                 cudaKernelNodeParams kp = {};
-                kp.func = sor2_kernel<R>(sv);
+                kp.func = sor2_kernel<R>(s2);
                 kp.gridDim = sor_grid;
-                kp.blockDim = dim3(sor_vbs(sv), 1, 1);
-                kp.sharedMemBytes = (unsigned)sor2_smem<R>(sv);
+                kp.blockDim = dim3(sor_vbs(s2), 1, 1);
+                kp.sharedMemBytes = (unsigned)sor2_smem<R>(s2);
                 kp.kernelParams = args;
                 cudaGraphNode_t kn;
                 CK(cudaGraphAddKernelNode(&kn, body, nullptr, 0, &kp));
@@ -785,7 +812,7 @@ struct Solver : Base {
         if (D == 2) {
             int maxr = sor_rounds();
             void *args[] = {(void *)&I, (void *)&h, (void *)&maxr, (void *)&r};
-            cudaLaunchKernel(sor2_kernel<R>(sv), sor_grid, dim3(sor_vbs(sv)), args, sor2_smem<R>(sv),
+            cudaLaunchKernel(sor2_kernel<R>(s2), sor_grid, dim3(sor_vbs(s2)), args, sor2_smem<R>(s2),
                              s);
         } else if (sv == 1) {
             int maxr = sor_rounds();

@@ -842,13 +842,22 @@ struct SorTile {
 //   K:   2      2     2      4      4      4      4      6      8
 //   BS:  256    256   256    256    256    512    512    512    512
 // (variants 7 and 8 exceed the shared memory of a block in double precision)
-constexpr int kSorVariants = 9;
-__host__ __device__ constexpr int sor_vtx(int v) { return (v == 1 || v == 6) ? 64 : (v == 2 ? 16 : 32); }
-__host__ __device__ constexpr int sor_vty(int v) {
-    return v == 1 ? 8 : ((v == 4 || v == 5 || v == 7) ? 32 : 16);
+// One more, not selectable: kSorSmall, 16 x 8 with the K of variant 0 (the same
+// iterates), which FP64 takes for variant 0 on grids of few tiles
+// (sor_variant_for).
+constexpr int kSorVariants = 9, kSorSmall = 9;
+__host__ __device__ constexpr int sor_vtx(int v) {
+    return (v == 1 || v == 6) ? 64 : ((v == 2 || v == kSorSmall) ? 16 : 32);
 }
-__host__ __device__ constexpr int sor_vk(int v) { return v == 8 ? 8 : (v == 7 ? 6 : (v >= 3 ? 4 : 2)); }
-__host__ __device__ constexpr int sor_vbs(int v) { return v >= 5 ? 512 : 256; }
+__host__ __device__ constexpr int sor_vty(int v) {
+    return (v == 1 || v == kSorSmall) ? 8 : ((v == 4 || v == 5 || v == 7) ? 32 : 16);
+}
+__host__ __device__ constexpr int sor_vk(int v) {
+    return v == 8 ? 8 : (v == 7 ? 6 : ((v >= 3 && v != kSorSmall) ? 4 : 2));
+}
+__host__ __device__ constexpr int sor_vbs(int v) {
+    return v == kSorSmall ? 128 : (v >= 5 ? 512 : 256);
+}
 
 // convergence of a round: the largest update of its last sweep is within
 // sor_tol of the largest value, or (single precision) the updates stopped
