@@ -51,7 +51,7 @@ UNIT = "MLUPS"
 #   sor: 32 B a sweep and cell in FP32 (psi, C, two right-hand sides, a, chi
 #     read; psi, C written: the count of a plain unblocked sweep), whatever
 #     the sweeps the blocked kernel runs in shared memory; the one-launch form
-#     (k_sorfuse2) also carries the grad group's fields and, of the surf
+#     (k_solve2, k_sorfuse2) also carries the grad group's fields and, of the surf
 #     group's, a and chi for the total (psi, C are the last sweep's) and the
 #     rescale's read and write of psi, C (7 + 2 + 4 fields)
 def alg_bytes_2d(group, storage, sweeps=0, fused_sor=False):
@@ -627,7 +627,7 @@ def main():
     sweeps, rounds = dg["sor_iters_psi"], max(dg["sor_rounds"], 1)
     hbm, src = peaks()
     sha = src_hash()
-    # the fused step: two launches (k_lbfd2, k_sorfuse2); else the fused
+    # the fused step: two launches (k_lbfd2 and k_solve2 or k_sorfuse2); else the fused
     # step, the gradient, one launch a round, the total and the rescale
     nk = s.kernel_count()
     sor_launches = 1 if nk == 2 else nk - 4

@@ -261,7 +261,7 @@ int lbs_step_result(lbs_ctx *c, double *out);
  * 256, 2 = 16x16 / 2 / 256, 3 = 32x16 / 4 / 256, 4 = 32x32 / 4 / 256,
  * 5 = 32x32 / 4 / 512, 6 = 64x16 / 4 / 512, 7 = 32x32 / 6 / 512,
  * 8 = 32x16 / 8 / 512 (7 and 8 exceed a block's shared memory in FP64 and
- * are refused there).  More sweeps a launch mean fewer launches and a wider
+ * are refused there; variant 0 takes 16x8 tiles on small FP64 grids).  More sweeps a launch mean fewer launches and a wider
  * halo (2 per sweep); the iterates, and so the results, do not depend on the
  * choice except through where the convergence test falls (after every
  * launch's sweeps).  With one launch a solve (lbs_set_sor_persistent) FP32 and
@@ -285,8 +285,9 @@ int lbs_set_sor_tile(lbs_ctx *c, int variant);
  * rounds are the same either way; the totals are summed in different
  * orders, so FP32 results agree to rounding.  3D contexts with SOR variant 0 in
  * FP32 arithmetic: every sweep of a solve in one cooperative launch (on) or the
- * half-sweeps as launches of their own (off): the same iterates.  A barrier that waits too long (about a second) reports
- * LBS_ETIMEOUT.  Errors: LBS_EINVAL (no context), LBS_ECUDA. */
+ * half-sweeps as launches of their own (off): the same iterates.  FP64 2D
+ * grids of more tiles than SMs are swept a launch a round either way.  A
+ * barrier that waits too long (about a second) reports LBS_ETIMEOUT.  Errors: LBS_EINVAL (no context), LBS_ECUDA. */
 int lbs_set_sor_persistent(lbs_ctx *c, int on);
 
 /* The most polls (about 64 ns each) a block of the one-launch SOR waits at
@@ -328,13 +329,16 @@ const char *lbs_last_error(const lbs_ctx *c);
 /* ------------------------------------------------------------------------
  * Batched sweep: n independent 2D instances (each its own lbs_params: grid,
  * Eotvos / Biot numbers, confinement; transport on) advanced together.
- * Each phase of the coupled step is one launch for the whole batch: a grid of
- * (SM count x resident blocks) blocks walks a work list of (instance, tile)
- * items.  The SOR rounds of all instances run in one CUDA-graph WHILE loop,
- * each instance with its own round counter and convergence test (Sec. 2.2
+ * In FP32 arithmetic the step up to the moments of t+1 is one launch an
+ * instance, side by side on streams of the batch between two events of its
+ * own, and the solves of all instances are one cooperative launch where their
+ * tiles fit the chip.  Other phases (and FP64) are one launch for the whole
+ * batch: a grid of (SM count x resident blocks) blocks walks a work list of
+ * (instance, tile) items, and the SOR rounds run in one CUDA-graph WHILE loop.
+ * Each instance has its own round counter and convergence test (Sec. 2.2
  * tolerance); a converged instance skips the remaining rounds.  One graph
  * holds 8 steps.  Results agree with n single-instance contexts to the
- * rounding of the storage type (the same per-cell bodies, compiled apart). */
+ * rounding of the storage type (the same bodies, compiled apart). */
 typedef struct lbs_batch lbs_batch;
 
 /* Device bytes of the instances' state for p[0..n-1] (0 on invalid input:
@@ -356,7 +360,7 @@ int lbs_batch_init_fields(lbs_batch *b, int k, const double *phi, const double *
                           const double *C, const double *u);
 
 /* Tile shapes: the cell phases run tx x ty thread blocks, one cell per
- * thread (tx*ty a multiple of 32, at most 1024); sor_tile selects the
+ * thread (the fused steps of FP32 arithmetic choose their own; tx*ty a multiple of 32, at most 1024); sor_tile selects the
  * blocked SOR tile and its sweeps a round as lbs_set_sor_tile (0..4).
  * Default 32 x 8, 0.  The cell tile does not change results; the SOR tile
  * only through where the convergence test falls. */
