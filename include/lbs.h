@@ -261,8 +261,8 @@ int lbs_step_result(lbs_ctx *c, double *out);
  * 256, 2 = 16x16 / 2 / 256, 3 = 32x16 / 4 / 256, 4 = 32x32 / 4 / 256,
  * 5 = 32x32 / 4 / 512, 6 = 64x16 / 4 / 512, 7 = 32x32 / 6 / 512,
  * 8 = 32x16 / 8 / 512 (7 and 8 exceed a block's shared memory in FP64 and
- * are refused there; variant 0 takes 16x8 tiles on small FP64 grids).  More sweeps a launch mean fewer launches and a wider
- * halo (2 per sweep); the iterates, and so the results, do not depend on the
+ * are refused there; variant 0 takes 16x8 tiles on small FP64 grids).  More
+ * sweeps a launch mean fewer launches and a wider halo (2 per sweep); the iterates, and so the results, do not depend on the
  * choice except through where the convergence test falls (after every
  * launch's sweeps).  With one launch a solve (lbs_set_sor_persistent) FP32 and
  * 16-bit grids that fit the GPU at once take tiles chosen for their size instead
@@ -287,7 +287,8 @@ int lbs_set_sor_tile(lbs_ctx *c, int variant);
  * FP32 arithmetic: every sweep of a solve in one cooperative launch (on) or the
  * half-sweeps as launches of their own (off): the same iterates.  FP64 2D
  * grids of more tiles than SMs are swept a launch a round either way.  A
- * barrier that waits too long (about a second) reports LBS_ETIMEOUT.  Errors: LBS_EINVAL (no context), LBS_ECUDA. */
+ * barrier that waits too long (about a second) reports LBS_ETIMEOUT.  Errors:
+ * LBS_EINVAL (no context), LBS_ECUDA. */
 int lbs_set_sor_persistent(lbs_ctx *c, int on);
 
 /* The most polls (about 64 ns each) a block of the one-launch SOR waits at
@@ -360,8 +361,8 @@ int lbs_batch_init_fields(lbs_batch *b, int k, const double *phi, const double *
                           const double *C, const double *u);
 
 /* Tile shapes: the cell phases run tx x ty thread blocks, one cell per
- * thread (the fused steps of FP32 arithmetic choose their own; tx*ty a multiple of 32, at most 1024); sor_tile selects the
- * blocked SOR tile and its sweeps a round as lbs_set_sor_tile (0..4).
+ * thread (tx*ty a multiple of 32, at most 1024; the fused steps of FP32
+ * arithmetic choose their own); sor_tile selects the blocked SOR tile and its sweeps a round as lbs_set_sor_tile (0..4).
  * Default 32 x 8, 0.  The cell tile does not change results; the SOR tile
  * only through where the convergence test falls. */
 int lbs_batch_set_tiles(lbs_batch *b, int tx, int ty, int sor_tile);

@@ -703,14 +703,14 @@ struct Solver : Base {
             ran[LBS_K_FORCE] = true;
             mark(s, LBS_K_FD);
             if (I.transport) {
-                L3::fd(I, grid, block, s, nullptr, nullptr);
+                L3::fd(I, s, nullptr, nullptr);
                 ran[LBS_K_FD] = true;
             }
             mark(s, LBS_K_COLLIDE);
             L3::collide(I, s);
             ran[LBS_K_COLLIDE] = true;
             mark(s, LBS_K_STREAM);
-            L3::stream(I, grid, block, s);
+            L3::stream(I, s);
             ran[LBS_K_STREAM] = true;
             mark(s, LBS_K_GRAD);
             L3::grad(I, s);
@@ -1161,7 +1161,7 @@ struct Solver : Base {
         if (D == 2)
             k_fd2<R><<<grid, block, 0, s>>>(I, dS, dB);
         else
-            L3::fd(I, grid, block, s, dS, dB);
+            L3::fd(I, s, dS, dB);
         r = launch_check();
         if (r) return r;
         struct {

@@ -24,10 +24,9 @@ struct Launch3 {
     static void moments(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s);
     static void grad(const Inst<R> &I, cudaStream_t s, int guess = 1);
     static void force(const Inst<R> &I, cudaStream_t s);
-    static void fd(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s, double *Sout,
-                   double *Bout);
+    static void fd(const Inst<R> &I, cudaStream_t s, double *Sout, double *Bout);
     static void collide(const Inst<R> &I, cudaStream_t s);
-    static void stream(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s);
+    static void stream(const Inst<R> &I, cudaStream_t s);
     static void diag(const Inst<R> &I, dim3 g, dim3 b, cudaStream_t s, int nblocks);
     // one red (colour 0) or black (colour 1) SOR half-sweep: variant 0 one
     // thread a cell (k_sor_rb3), variants 2 and 3 column marching through 8

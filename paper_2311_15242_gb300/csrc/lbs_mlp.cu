@@ -89,10 +89,10 @@ __global__ void k_copy_weights(const float *p, Shape s, int E, float *W) {
 // wavefronts a warp each, for 16 C multiply-adds: at C = 2 the loads take 12
 // cycles of the SM's shared memory and the multiply-adds 8 of its FP32 pipes.
 // (8 x 8 tiles would balance them, but leave 8 warps an SM, too few to hide the
-// loads: 40,000 rows 0.44 -> 0.54 ms.)  ROWS = 64 (C = 2) serves inference, where there are enough
-// rows to fill the chip; ROWS = 16 (C = 1) serves training and short
-// batches, where the minibatch of every member must spread over many blocks;
-// its threads split k in two halves, since 128 threads alone leave the
+// loads: 40,000 rows 0.44 -> 0.54 ms.)  ROWS = 64 (C = 2) serves inference, where
+// there are enough rows to fill the chip; ROWS = 16 (C = 1) serves training and
+// short batches, where the minibatch of every member must spread over many
+// blocks; its threads split k in two halves, since 128 threads alone leave the
 // schedulers idle.
 // ---------------------------------------------------------------------------
 template <int ROWS>
