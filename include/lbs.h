@@ -262,15 +262,16 @@ int lbs_step_result(lbs_ctx *c, double *out);
  * 5 = 32x32 / 4 / 512, 6 = 64x16 / 4 / 512, 7 = 32x32 / 6 / 512,
  * 8 = 32x16 / 8 / 512 (7 and 8 exceed a block's shared memory in FP64 and
  * are refused there; variant 0 takes 16x8 tiles on small FP64 grids).  More
- * sweeps a launch mean fewer launches and a wider halo (2 per sweep); the iterates, and so the results, do not depend on the
- * choice except through where the convergence test falls (after every
- * launch's sweeps).  With one launch a solve (lbs_set_sor_persistent) FP32 and
- * 16-bit grids that fit the GPU at once take tiles chosen for their size instead
- * (periodic x: even nx); the variant then sets the 2 or 4 sweeps between
- * convergence tests.  3D contexts: 0 = a red and a black half-sweep a sweep, in
- * place, one thread a cell, or the same sweeps in one launch a solve
- * (lbs_set_sor_persistent) (default), 1 = one full red-black sweep a launch with
- * 32x8 tiles marching through 16-plane chunks of z in shared memory, 2 and
+ * sweeps a launch mean fewer launches and a wider halo (2 per sweep); the
+ * iterates, and so the results, do not depend on the choice except through
+ * where the convergence test falls (after every launch's sweeps).  With one
+ * launch a solve (lbs_set_sor_persistent) FP32 and 16-bit grids that fit the
+ * GPU at once take tiles chosen for their size instead (periodic x: even nx);
+ * the variant then sets the 2 or 4 sweeps between convergence tests.  3D
+ * contexts: 0 = a red and a black half-sweep a sweep, in place, one thread a
+ * cell, or the same sweeps in one launch a solve (lbs_set_sor_persistent)
+ * (default), 1 = one full red-black sweep a launch with 32x8 tiles marching
+ * through 16-plane chunks of z in shared memory, 2 and
  * 3 = the half-sweeps of 0 with each thread marching a cell pair through 8
  * or 4 planes of z.  Errors: LBS_EINVAL. */
 int lbs_set_sor_tile(lbs_ctx *c, int variant);
@@ -362,7 +363,8 @@ int lbs_batch_init_fields(lbs_batch *b, int k, const double *phi, const double *
 
 /* Tile shapes: the cell phases run tx x ty thread blocks, one cell per
  * thread (tx*ty a multiple of 32, at most 1024; the fused steps of FP32
- * arithmetic choose their own); sor_tile selects the blocked SOR tile and its sweeps a round as lbs_set_sor_tile (0..4).
+ * arithmetic choose their own); sor_tile selects the blocked SOR tile and its
+ * sweeps a round as lbs_set_sor_tile (0..4).
  * Default 32 x 8, 0.  The cell tile does not change results; the SOR tile
  * only through where the convergence test falls. */
 int lbs_batch_set_tiles(lbs_batch *b, int tx, int ty, int sor_tile);

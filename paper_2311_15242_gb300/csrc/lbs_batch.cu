@@ -8,15 +8,16 @@
 // work list of (instance, tile) items, copies the instance's descriptor into
 // shared memory when the instance changes and runs the same per-cell bodies as
 // the single-instance kernels; FP64, bound by its arithmetic, of which a tile's
-// halo would be a quarter more, takes all phases that way.  The SOR rounds of all instances share one WHILE node: each
-// instance keeps its own round counter, convergence test and ping-pong
-// parity, a converged instance's tiles skip the remaining rounds, and the
-// loop ends when no instance is still iterating.  In FP32 arithmetic, where
-// every instance's tiles fit the chip at once (k_solve2's tiles, at most one an
-// SM), the gradient, the solve, the total and the rescale of all instances are
-// one cooperative launch instead (kb_solve2).  A CUDA graph holds several
-// whole steps.  The cell-tile shape (block shape) and the SOR tile are
-// chosen at run time (lbs_batch_set_tiles; the autotuner picks them).
+// halo would be a quarter more, takes all phases that way.  The SOR rounds of
+// all instances share one WHILE node: each instance keeps its own round
+// counter, convergence test and ping-pong parity, a converged instance's tiles
+// skip the remaining rounds, and the loop ends when no instance is still
+// iterating.  In FP32 arithmetic, where every instance's tiles fit the chip at
+// once (k_solve2's tiles, at most one an SM), the gradient, the solve, the
+// total and the rescale of all instances are one cooperative launch instead
+// (kb_solve2).  A CUDA graph holds several whole steps.  The cell-tile shape
+// (block shape) and the SOR tile are chosen at run time (lbs_batch_set_tiles;
+// the autotuner picks them).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -258,54 +258,54 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 5 : 2) k_force3(Inst<R> 
     __syncthreads();
 #pragma unroll 1
     for (int k = 0; k < T::TZ / 2; k++) {
-    LBS_TILE_CELL3(k)
-    // (the cell's own values first: one wait for memory a cell)
-    const R a = I.a[c], rR = I.rhoR[c], rB = I.rhoB[c];
-    const R jx = I.jx[c], jy = I.jy[c], jz = I.jz[c];
-    R divn = R(0), dpx = R(0), dpy = R(0), dpz = R(0);
+        LBS_TILE_CELL3(k)
+        // (the cell's own values first: one wait for memory a cell)
+        const R a = I.a[c], rR = I.rhoR[c], rB = I.rhoB[c];
+        const R jx = I.jx[c], jy = I.jy[c], jz = I.jz[c];
+        R divn = R(0), dpx = R(0), dpy = R(0), dpz = R(0);
 #pragma unroll
-    for (int i = 1; i < Q19; i++) {
-        const int j = q + T::off(ex19(i), ey19(i), ez19(i));
-        R s = R(0);
-        if (ex19(i)) s += R(ex19(i)) * g3[0][j];
-        if (ey19(i)) s += R(ey19(i)) * g3[1][j];
-        if (ez19(i)) s += R(ez19(i)) * g3[2][j];
-        divn -= w19<R>(i) * s * inv3[j];
-        const R p = w19<R>(i) * psi3[j];
-        if (ex19(i)) dpx += R(ex19(i)) * p;
-        if (ey19(i)) dpy += R(ey19(i)) * p;
-        if (ez19(i)) dpz += R(ez19(i)) * p;
-    }
-    const R kappa = -R(3) * divn;
-    dpx *= R(3);
-    dpy *= R(3);
-    dpz *= R(3);
-    const R gx = g3[0][q], gy = g3[1][q], gz = g3[2][q];
-    R sigma, mco, Fx, Fy, Fz;
-    if (eos(I, psi3[q], sigma, mco)) {
-        const R inv = inv3[q];
-        const R nx = -gx * inv, ny = -gy * inv, nz = -gz * inv;
-        const R ndp = nx * dpx + ny * dpy + nz * dpz;
-        Fx = -R(0.5) * sigma * kappa * gx - R(0.5) * a * mco * (dpx - ndp * nx);
-        Fy = -R(0.5) * sigma * kappa * gy - R(0.5) * a * mco * (dpy - ndp * ny);
-        Fz = -R(0.5) * sigma * kappa * gz - R(0.5) * a * mco * (dpz - ndp * nz);
-    } else {
-        Fx = -R(0.5) * I.sigma_min * kappa * gx;
-        Fy = -R(0.5) * I.sigma_min * kappa * gy;
-        Fz = -R(0.5) * I.sigma_min * kappa * gz;
-    }
-    const R rho = rR + rB;
-    const R drb = rR + (rB - I.rhoB0);
-    Fx += drb * I.g[0];
-    Fy += drb * I.g[1];
-    Fz += drb * I.g[2];
-    I.Fx[c] = Fx;
-    I.Fy[c] = Fy;
-    I.Fz[c] = Fz;
-    const R irho = fdiv(R(1), rho);
-    I.ux[c] = (jx + R(0.5) * Fx) * irho;
-    I.uy[c] = (jy + R(0.5) * Fy) * irho;
-    I.uz[c] = (jz + R(0.5) * Fz) * irho;
+        for (int i = 1; i < Q19; i++) {
+            const int j = q + T::off(ex19(i), ey19(i), ez19(i));
+            R s = R(0);
+            if (ex19(i)) s += R(ex19(i)) * g3[0][j];
+            if (ey19(i)) s += R(ey19(i)) * g3[1][j];
+            if (ez19(i)) s += R(ez19(i)) * g3[2][j];
+            divn -= w19<R>(i) * s * inv3[j];
+            const R p = w19<R>(i) * psi3[j];
+            if (ex19(i)) dpx += R(ex19(i)) * p;
+            if (ey19(i)) dpy += R(ey19(i)) * p;
+            if (ez19(i)) dpz += R(ez19(i)) * p;
+        }
+        const R kappa = -R(3) * divn;
+        dpx *= R(3);
+        dpy *= R(3);
+        dpz *= R(3);
+        const R gx = g3[0][q], gy = g3[1][q], gz = g3[2][q];
+        R sigma, mco, Fx, Fy, Fz;
+        if (eos(I, psi3[q], sigma, mco)) {
+            const R inv = inv3[q];
+            const R nx = -gx * inv, ny = -gy * inv, nz = -gz * inv;
+            const R ndp = nx * dpx + ny * dpy + nz * dpz;
+            Fx = -R(0.5) * sigma * kappa * gx - R(0.5) * a * mco * (dpx - ndp * nx);
+            Fy = -R(0.5) * sigma * kappa * gy - R(0.5) * a * mco * (dpy - ndp * ny);
+            Fz = -R(0.5) * sigma * kappa * gz - R(0.5) * a * mco * (dpz - ndp * nz);
+        } else {
+            Fx = -R(0.5) * I.sigma_min * kappa * gx;
+            Fy = -R(0.5) * I.sigma_min * kappa * gy;
+            Fz = -R(0.5) * I.sigma_min * kappa * gz;
+        }
+        const R rho = rR + rB;
+        const R drb = rR + (rB - I.rhoB0);
+        Fx += drb * I.g[0];
+        Fy += drb * I.g[1];
+        Fz += drb * I.g[2];
+        I.Fx[c] = Fx;
+        I.Fy[c] = Fy;
+        I.Fz[c] = Fz;
+        const R irho = fdiv(R(1), rho);
+        I.ux[c] = (jx + R(0.5) * Fx) * irho;
+        I.uy[c] = (jy + R(0.5) * Fy) * irho;
+        I.uz[c] = (jz + R(0.5) * Fz) * irho;
     }
 }
 
@@ -406,140 +406,140 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_collide3(Inst<R
     __syncthreads();
 #pragma unroll 1
     for (int k = 0; k < T::TZ / 2; k++) {
-    LBS_TILE_CELL3(k)
-    R fT[Q19], fM[Q19];
-    const int fl = I.flag[c];
+        LBS_TILE_CELL3(k)
+        R fT[Q19], fM[Q19];
+        const int fl = I.flag[c];
 #pragma unroll
-    for (int i = 0; i < Q19; i++) {
-        fT[i] = ldq<R, P>(I, I.fT, I.fT0, i, c);
-        fM[i] = ldq<R, P>(I, I.fM, I.fM0, i, c);
-    }
-    const Mom3<R> mo = moments19(I, fT, fM, fl);
-    const R rR = mo.rR, rB = mo.rB;
-    const R rmin = fl ? rB : rR;
-    const R devmaj = I.dsh[fl] + (mo.drho - rmin);
-    const R rho = rR + rB;
-    const R ux = u3[0][q], uy = u3[1][q], uz = u3[2][q];
-    const R Fx = I.Fx[c], Fy = I.Fy[c], Fz = I.Fz[c];
+        for (int i = 0; i < Q19; i++) {
+            fT[i] = ldq<R, P>(I, I.fT, I.fT0, i, c);
+            fM[i] = ldq<R, P>(I, I.fM, I.fM0, i, c);
+        }
+        const Mom3<R> mo = moments19(I, fT, fM, fl);
+        const R rR = mo.rR, rB = mo.rB;
+        const R rmin = fl ? rB : rR;
+        const R devmaj = I.dsh[fl] + (mo.drho - rmin);
+        const R rho = rR + rB;
+        const R ux = u3[0][q], uy = u3[1][q], uz = u3[2][q];
+        const R Fx = I.Fx[c], Fy = I.Fy[c], Fz = I.Fz[c];
 
-    // d_a(rho^k u_a), isotropic stencil
-    R dR[3] = {R(0), R(0), R(0)}, dB[3] = {R(0), R(0), R(0)};
+        // d_a(rho^k u_a), isotropic stencil
+        R dR[3] = {R(0), R(0), R(0)}, dB[3] = {R(0), R(0), R(0)};
 #pragma unroll
-    for (int i = 1; i < Q19; i++) {
-        const int j = q + T::off(ex19(i), ey19(i), ez19(i));
-        const int e[3] = {ex19(i), ey19(i), ez19(i)};
-        const R r1 = w19<R>(i) * rho3[0][j], r2 = w19<R>(i) * rho3[1][j];
+        for (int i = 1; i < Q19; i++) {
+            const int j = q + T::off(ex19(i), ey19(i), ez19(i));
+            const int e[3] = {ex19(i), ey19(i), ez19(i)};
+            const R r1 = w19<R>(i) * rho3[0][j], r2 = w19<R>(i) * rho3[1][j];
 #pragma unroll
-        for (int a = 0; a < 3; a++)
-            if (e[a]) {
-                const R v = u3[a][j];
-                dR[a] += R(e[a]) * r1 * v;
-                dB[a] += R(e[a]) * r2 * v;
-            }
-    }
-    const R cR = R(1) - R(1.5) * (R(1) - I.alphaR), cB = R(1) - R(1.5) * (R(1) - I.alphaB);
-    const R Qx = R(3) * (cR * dR[0] + cB * dB[0]);
-    const R Qy = R(3) * (cR * dR[1] + cB * dB[1]);
-    const R Qz = R(3) * (cR * dR[2] + cB * dB[2]);
+            for (int a = 0; a < 3; a++)
+                if (e[a]) {
+                    const R v = u3[a][j];
+                    dR[a] += R(e[a]) * r1 * v;
+                    dB[a] += R(e[a]) * r2 * v;
+                }
+        }
+        const R cR = R(1) - R(1.5) * (R(1) - I.alphaR), cB = R(1) - R(1.5) * (R(1) - I.alphaB);
+        const R Qx = R(3) * (cR * dR[0] + cB * dB[0]);
+        const R Qy = R(3) * (cR * dR[1] + cB * dB[1]);
+        const R Qz = R(3) * (cR * dR[2] + cB * dB[2]);
 
-    // moments of the shifted total populations (rows 4-18)
-    R mT[Q19];
+        // moments of the shifted total populations (rows 4-18)
+        R mT[Q19];
 #pragma unroll
-    for (int j = 4; j < Q19; j++) {
-        R s = R(0);
+        for (int j = 4; j < Q19; j++) {
+            R s = R(0);
 #pragma unroll
-        for (int i = 0; i < Q19; i++)
-            if (m19(j, i) != 0) s += R(m19(j, i)) * fT[i];
-        mT[j] = s;
-    }
-    const R Pk = rR * I.cs2R + rB * I.cs2B;
-    const R dP = fl == 0 ? devmaj * I.cs2B + rR * I.cs2R : devmaj * I.cs2R + rB * I.cs2B;
-    const R xx = ux * ux, yy = uy * uy, zz = uz * uz, u2 = xx + yy + zz;
-    R neq[Q19];
-    neq[4] = mT[4] - R(3) * dP - rho * u2 + I.mcor1[fl];
-    neq[5] = mT[5] - rho * (R(2) * xx - yy - zz);
-    neq[6] = mT[6] - rho * (yy - zz);
-    neq[7] = mT[7] - rho * ux * uy;
-    neq[8] = mT[8] - rho * ux * uz;
-    neq[9] = mT[9] - rho * uy * uz;
-    neq[10] = mT[10] - Pk * uy;
-    neq[11] = mT[11] - Pk * ux;
-    neq[12] = mT[12] - Pk * uz;
-    neq[13] = mT[13] - Pk * ux;
-    neq[14] = mT[14] - Pk * uz;
-    neq[15] = mT[15] - Pk * uy;
-    const R d3 = dP / R(3) - I.mcor2[fl];
-    neq[16] = mT[16] - d3 - rho * (xx + yy - zz) / R(6);
-    neq[17] = mT[17] - d3 - rho * (xx + zz - yy) / R(6);
-    neq[18] = mT[18] - d3 - rho * (yy + zz - xx) / R(6);
+            for (int i = 0; i < Q19; i++)
+                if (m19(j, i) != 0) s += R(m19(j, i)) * fT[i];
+            mT[j] = s;
+        }
+        const R Pk = rR * I.cs2R + rB * I.cs2B;
+        const R dP = fl == 0 ? devmaj * I.cs2B + rR * I.cs2R : devmaj * I.cs2R + rB * I.cs2B;
+        const R xx = ux * ux, yy = uy * uy, zz = uz * uz, u2 = xx + yy + zz;
+        R neq[Q19];
+        neq[4] = mT[4] - R(3) * dP - rho * u2 + I.mcor1[fl];
+        neq[5] = mT[5] - rho * (R(2) * xx - yy - zz);
+        neq[6] = mT[6] - rho * (yy - zz);
+        neq[7] = mT[7] - rho * ux * uy;
+        neq[8] = mT[8] - rho * ux * uz;
+        neq[9] = mT[9] - rho * uy * uz;
+        neq[10] = mT[10] - Pk * uy;
+        neq[11] = mT[11] - Pk * ux;
+        neq[12] = mT[12] - Pk * uz;
+        neq[13] = mT[13] - Pk * ux;
+        neq[14] = mT[14] - Pk * uz;
+        neq[15] = mT[15] - Pk * uy;
+        const R d3 = dP / R(3) - I.mcor2[fl];
+        neq[16] = mT[16] - d3 - rho * (xx + yy - zz) / R(6);
+        neq[17] = mT[17] - d3 - rho * (xx + zz - yy) / R(6);
+        neq[18] = mT[18] - d3 - rho * (yy + zz - xx) / R(6);
 
-    // s_v from the mixture viscosity (Eq. 43)
-    const R rN = colour_fn(I, rR, rB);
-    const R inv_mu = (R(1) + rN) * I.inv_2muR + (R(1) - rN) * I.inv_2muB;
-    const R sv = fdiv(R(1), R(0.5) + fdiv(R(1), inv_mu * Pk));
-    const R uF = ux * Fx + uy * Fy + uz * Fz;
-    const R xF = ux * Fx, yF = uy * Fy, zF = uz * Fz;
-    R dm[Q19];
-    dm[0] = R(0);
-    dm[1] = Fx;
-    dm[2] = Fy;
-    dm[3] = Fz;
-    dm[4] = -neq[4] + R(0.5) * ((Qx + Qy + Qz) + R(2) * uF);
-    const R hv = R(1) - R(0.5) * sv;
-    dm[5] = -sv * neq[5] + hv * ((R(2) * Qx - Qy - Qz) + (R(4) * xF - R(2) * yF - R(2) * zF));
-    dm[6] = -sv * neq[6] + hv * ((Qy - Qz) + (R(2) * yF - R(2) * zF));
-    dm[7] = -sv * neq[7] + hv * (ux * Fy + uy * Fx);
-    dm[8] = -sv * neq[8] + hv * (ux * Fz + uz * Fx);
-    dm[9] = -sv * neq[9] + hv * (uy * Fz + uz * Fy);
-    const R t3 = R(0.5) / R(3);
-    dm[10] = -neq[10] + t3 * Fy;
-    dm[11] = -neq[11] + t3 * Fx;
-    dm[12] = -neq[12] + t3 * Fz;
-    dm[13] = -neq[13] + t3 * Fx;
-    dm[14] = -neq[14] + t3 * Fz;
-    dm[15] = -neq[15] + t3 * Fy;
-    const R uF3 = uF / R(3);
-    dm[16] = -neq[16] + R(0.5) * (xF + yF - uF3);
-    dm[17] = -neq[17] + R(0.5) * (xF + zF - uF3);
-    dm[18] = -neq[18] + R(0.5) * (yF + zF - uF3);
-    R df[Q19];
-    minv19<R>(dm, df);
+        // s_v from the mixture viscosity (Eq. 43)
+        const R rN = colour_fn(I, rR, rB);
+        const R inv_mu = (R(1) + rN) * I.inv_2muR + (R(1) - rN) * I.inv_2muB;
+        const R sv = fdiv(R(1), R(0.5) + fdiv(R(1), inv_mu * Pk));
+        const R uF = ux * Fx + uy * Fy + uz * Fz;
+        const R xF = ux * Fx, yF = uy * Fy, zF = uz * Fz;
+        R dm[Q19];
+        dm[0] = R(0);
+        dm[1] = Fx;
+        dm[2] = Fy;
+        dm[3] = Fz;
+        dm[4] = -neq[4] + R(0.5) * ((Qx + Qy + Qz) + R(2) * uF);
+        const R hv = R(1) - R(0.5) * sv;
+        dm[5] = -sv * neq[5] + hv * ((R(2) * Qx - Qy - Qz) + (R(4) * xF - R(2) * yF - R(2) * zF));
+        dm[6] = -sv * neq[6] + hv * ((Qy - Qz) + (R(2) * yF - R(2) * zF));
+        dm[7] = -sv * neq[7] + hv * (ux * Fy + uy * Fx);
+        dm[8] = -sv * neq[8] + hv * (ux * Fz + uz * Fx);
+        dm[9] = -sv * neq[9] + hv * (uy * Fz + uz * Fy);
+        const R t3 = R(0.5) / R(3);
+        dm[10] = -neq[10] + t3 * Fy;
+        dm[11] = -neq[11] + t3 * Fx;
+        dm[12] = -neq[12] + t3 * Fz;
+        dm[13] = -neq[13] + t3 * Fx;
+        dm[14] = -neq[14] + t3 * Fz;
+        dm[15] = -neq[15] + t3 * Fy;
+        const R uF3 = uF / R(3);
+        dm[16] = -neq[16] + R(0.5) * (xF + yF - uF3);
+        dm[17] = -neq[17] + R(0.5) * (xF + zF - uF3);
+        dm[18] = -neq[18] + R(0.5) * (yF + zF - uF3);
+        R df[Q19];
+        minv19<R>(dm, df);
 
-    R post[Q19];
-    CSum<R> rdc;
+        R post[Q19];
+        CSum<R> rdc;
 #pragma unroll
-    for (int i = 0; i < Q19; i++) {
-        post[i] = fT[i] + df[i];
-        rdc.add(shift_of(I, i, fl) + post[i]);
-    }
-    const R rdag = rdc.value();
-    // recolouring: segregation weight f_i^eq(rho, 0)/rho = w_i 3 P / rho for
-    // the moving directions (the rest equilibrium of Eq. 40: rho - 2P at rest,
-    // P/6 on the axes, P/12 on the diagonals)
-    const R ggx = I.gx[c], ggy = I.gy[c], ggz = I.gz[c];
-    const R seg = I.beta * rR * rB * R(3) * Pk *
-                  frsq(ggx * ggx + ggy * ggy + ggz * ggz + I.eps_n * I.eps_n) *
-                  fdiv(R(1), rho * rho);
-    const R fr = fdiv(rmin, rdag);
-    const R sg = fl ? R(-1) : R(1);
-    // moving populations as stored; the rest populations close the cell's
-    // total and minority mass on the pre-collision values (see k_collide2)
-    CSum<R> sT, sM;
-    const unsigned int rk = rest_key(c, rest_salt(0, I.ctl->step)), rs = pop_seed(rk);
+        for (int i = 0; i < Q19; i++) {
+            post[i] = fT[i] + df[i];
+            rdc.add(shift_of(I, i, fl) + post[i]);
+        }
+        const R rdag = rdc.value();
+        // recolouring: segregation weight f_i^eq(rho, 0)/rho = w_i 3 P / rho for
+        // the moving directions (the rest equilibrium of Eq. 40: rho - 2P at rest,
+        // P/6 on the axes, P/12 on the diagonals)
+        const R ggx = I.gx[c], ggy = I.gy[c], ggz = I.gz[c];
+        const R seg = I.beta * rR * rB * R(3) * Pk *
+                      frsq(ggx * ggx + ggy * ggy + ggz * ggz + I.eps_n * I.eps_n) *
+                      fdiv(R(1), rho * rho);
+        const R fr = fdiv(rmin, rdag);
+        const R sg = fl ? R(-1) : R(1);
+        // moving populations as stored; the rest populations close the cell's
+        // total and minority mass on the pre-collision values (see k_collide2)
+        CSum<R> sT, sM;
+        const unsigned int rk = rest_key(c, rest_salt(0, I.ctl->step)), rs = pop_seed(rk);
 #pragma unroll
-    for (int i = 1; i < Q19; i++) {
-        R eg = R(0);
-        if (ex19(i)) eg += R(ex19(i)) * ggx;
-        if (ey19(i)) eg += R(ey19(i)) * ggy;
-        if (ez19(i)) eg += R(ez19(i)) * ggz;
-        const R segi = seg * w19<R>(i) * eg;
-        sT.add(stq_r<R, P>(I, I.gT, i, c, post[i], pop_r(rs, 2 * i)));
-        sM.add(stq_r<R, P>(I, I.gM, i, c, fr * (I.shift[i] + post[i]) + sg * segi,
-                           pop_r(rs, 2 * i + 1)));
-    }
-    I.gT0[c] = rest_close(mo.dr_s, mo.dr_c, sT.s, sT.c, R(0), rest_u(rk, 0));
-    I.gM0[c] = rest_close(mo.rm_s, mo.rm_c, sM.s, sM.c, R(0), rest_u(rk, 1));
-    I.gflag[c] = (uint8_t)fl;
+        for (int i = 1; i < Q19; i++) {
+            R eg = R(0);
+            if (ex19(i)) eg += R(ex19(i)) * ggx;
+            if (ey19(i)) eg += R(ey19(i)) * ggy;
+            if (ez19(i)) eg += R(ez19(i)) * ggz;
+            const R segi = seg * w19<R>(i) * eg;
+            sT.add(stq_r<R, P>(I, I.gT, i, c, post[i], pop_r(rs, 2 * i)));
+            sM.add(stq_r<R, P>(I, I.gM, i, c, fr * (I.shift[i] + post[i]) + sg * segi,
+                               pop_r(rs, 2 * i + 1)));
+        }
+        I.gT0[c] = rest_close(mo.dr_s, mo.dr_c, sT.s, sT.c, R(0), rest_u(rk, 0));
+        I.gM0[c] = rest_close(mo.rm_s, mo.rm_c, sM.s, sM.c, R(0), rest_u(rk, 1));
+        I.gflag[c] = (uint8_t)fl;
     }
 }
 
@@ -560,43 +560,43 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_stream3(Inst<R>
     R t[Q19], m[Q19];
     int slow = 0;
     {
-    const Ax X = make_ax(x, I.nx, I.wall[0], 1), Y = make_ax(y, I.ny, I.wall[1], 2),
-             Z = make_ax(z, I.nz, I.wall[2], 4);
-    t[0] = I.gT0[c];
-    m[0] = I.gM0[c];
-    const int near = X.r[1] | X.r[3] | Y.r[1] | Y.r[3] | Z.r[1] | Z.r[3];
-    if (!__any_sync(__activemask(), near)) {
-        // no link of the warp's cells crosses a boundary: plain pulls (most
-        // warps; a third of the other form's instructions)
+        const Ax X = make_ax(x, I.nx, I.wall[0], 1), Y = make_ax(y, I.ny, I.wall[1], 2),
+                 Z = make_ax(z, I.nz, I.wall[2], 4);
+        t[0] = I.gT0[c];
+        m[0] = I.gM0[c];
+        const int near = X.r[1] | X.r[3] | Y.r[1] | Y.r[3] | Z.r[1] | Z.r[3];
+        if (!__any_sync(__activemask(), near)) {
+            // no link of the warp's cells crosses a boundary: plain pulls (most
+            // warps; a third of the other form's instructions)
 #pragma unroll
-        for (int i = 1; i < Q19; i++) {
-            int refl, sx, sy, sz;
-            const unsigned j = nbx3(I, X, Y, Z, -ex19(i), -ey19(i), -ez19(i), refl, sx, sy, sz);
-            const long long k = (long long)i * I.plane + j;
-            t[i] = ldp<R, P>(I, I.gT, k);
-            m[i] = ldp<R, P>(I, I.gM, k);
-            slow |= I.gflag[j] ^ flc;
-        }
-    } else {
-        // a link that crosses a wall reflects the cell's own opposite
-        // population (branch-free, so that every load of the loop can be in
-        // flight at once)
+            for (int i = 1; i < Q19; i++) {
+                int refl, sx, sy, sz;
+                const unsigned j = nbx3(I, X, Y, Z, -ex19(i), -ey19(i), -ez19(i), refl, sx, sy, sz);
+                const long long k = (long long)i * I.plane + j;
+                t[i] = ldp<R, P>(I, I.gT, k);
+                m[i] = ldp<R, P>(I, I.gM, k);
+                slow |= I.gflag[j] ^ flc;
+            }
+        } else {
+            // a link that crosses a wall reflects the cell's own opposite
+            // population (branch-free, so that every load of the loop can be in
+            // flight at once)
 #pragma unroll
-        for (int i = 1; i < Q19; i++) {
-            int refl, sx, sy, sz;
-            const unsigned j = nbx3(I, X, Y, Z, -ex19(i), -ey19(i), -ez19(i), refl, sx, sy, sz);
-            const int bb = refl & I.bbmask;  // mirror planes: the mirrored source
-            const unsigned src = bb ? c : j;
-            const int dir = bb ? opp19(i) : (MIRROR ? mir19(i, refl) : i);
-            const long long k = (long long)dir * I.plane + src;
-            t[i] = ldp<R, P>(I, I.gT, k);
-            m[i] = ldp<R, P>(I, I.gM, k);
-            // (a static wall returns the cell's own opposite population
-            // unchanged: the fast path's plain move; a moving wall adds its
-            // momentum term)
-            slow |= (I.gflag[src] ^ flc) | (bb & I.mvmask);
+            for (int i = 1; i < Q19; i++) {
+                int refl, sx, sy, sz;
+                const unsigned j = nbx3(I, X, Y, Z, -ex19(i), -ey19(i), -ez19(i), refl, sx, sy, sz);
+                const int bb = refl & I.bbmask;  // mirror planes: the mirrored source
+                const unsigned src = bb ? c : j;
+                const int dir = bb ? opp19(i) : (MIRROR ? mir19(i, refl) : i);
+                const long long k = (long long)dir * I.plane + src;
+                t[i] = ldp<R, P>(I, I.gT, k);
+                m[i] = ldp<R, P>(I, I.gM, k);
+                // (a static wall returns the cell's own opposite population
+                // unchanged: the fast path's plain move; a moving wall adds its
+                // momentum term)
+                slow |= (I.gflag[src] ^ flc) | (bb & I.mvmask);
+            }
         }
-    }
     }
     // 2. fast path: every population moves unchanged; the cell keeps its
     //    flag unless its minority colour has become the majority
