@@ -9,6 +9,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "lbs_log.cuh"
+
 namespace lbs {
 
 // ---------------------------------------------------------------------------
@@ -573,49 +575,20 @@ __device__ __forceinline__ void ghost_u3(const Inst<R> &I, int refl, int sx, int
     }
 }
 
-// ---------------------------------------------------------------------------
-// log(1 + x) of the equation of state.  In single precision by the argument
-// reduction and series of Cody and Waite (Software Manual for the Elementary
-// Functions, 1980), carried so that only the last rounding counts:
-//   1 + x = u + err exactly, u = 2^e (1 + f) with 2/3 <= 1 + f < 4/3,
-//   log(1 + x) = e ln 2 + f - f^2/2 + f^3 p(f) + 2^-e err / (1 + f),
-// p by Chebyshev interpolation of its Taylor series.  Below x = -1/2 the sum
-// 1 + x is exact and the error at most 0.52 ulp, above 0.82 ulp; the
-// logarithm near saturation (psi / psi_inf > 1/2) needs that accuracy and
-// was taken in double precision, whose 60-odd instructions run at 1/64 of the
-// single precision rate here: with half the cells above 1/2 the force kernel of
-// a 256 x 128 x 128 grid took 165 us, now 77.  (CUDA's log1pf was measured
-// at up to 0.89 ulp over the same arguments.)
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ double log1p_r(double x) { return log1p(x); }
-__device__ __forceinline__ float log1p_r(float x) {
-    if (!(x > -1.0f && x <= 1.0f)) return log1pf(x);
-    const float u = 1.0f + x, err = x - (u - 1.0f);
-    const int i = __float_as_int(u) - 0x3F2AAAAB, e = i >> 23;
-    const float f = __int_as_float((i & 0x7FFFFF) + 0x3F2AAAAB) - 1.0f;
-    const float fl = err * __int_as_float((127 - e) << 23), ef = float(e);
-    float p = 0.11622506f;
-    p = fmaf(p, f, -0.12432694f);
-    p = fmaf(p, f, 0.10851078f);
-    p = fmaf(p, f, -0.12286765f);
-    p = fmaf(p, f, 0.14296326f);
-    p = fmaf(p, f, -0.16673420f);
-    p = fmaf(p, f, 0.19999850f);
-    p = fmaf(p, f, -0.24999943f);
-    p = fmaf(p, f, 0.33333334f);
-    const float f2 = __fmul_rn(f, f);
-    const float hi = __fmul_rn(ef, 0x1.62E4p-1f);  // (ln 2 to 16 bits: exact)
-    const float s = __fadd_rn(hi, f), e1 = f - (s - hi);
-    const float s2 = fmaf(-0.5f, f2, s), e2 = fmaf(-0.5f, f2, s - s2);
-    float t = fmaf(ef, 1.4286068e-6f, fmaf(-f, fl, fl));
-    t = fmaf(-0.5f, fmaf(f, f, -f2), t);
-    t = fmaf(f2 * f, p, t);
-    return s2 + (e2 + (e1 + t));
+// log(1 + x) in double precision, rounded (a call: it is rare, and its code
+// stays out of the callers')
+static __device__ __noinline__ float log1p_double(float x) { return float(log1p(double(x))); }
+__device__ __forceinline__ double log1p_eos(double x) { return log1p(x); }
+__device__ __forceinline__ float log1p_eos(float x) {
+    if (!(x < -0.5f)) return log1pf(x);
+    float r;
+    return x > -1.0f && log1p_pair(x, r) ? r : log1p_double(x);
 }
 
 // ---------------------------------------------------------------------------
 // Equation of state (Eq. 8) and the Marangoni coefficient -d sigma/d psi of
-// Eq. 9.  Above the CMC sigma = sigma_min and the coefficient is 0.
+// Eq. 9.  Above the CMC sigma = sigma_min and the coefficient is 0.  The
+// logarithm is that of double precision near saturation (psi/psi_inf > 1/2).
 // ---------------------------------------------------------------------------
 template <typename R>
 __device__ __forceinline__ bool eos(const Inst<R> &I, R psi, R &sigma, R &mcoef) {
@@ -630,7 +603,7 @@ __device__ __forceinline__ bool eos(const Inst<R> &I, R psi, R &sigma, R &mcoef)
         return true;
     }
     if (psi < I.cmc) {
-        const R lg = log1p_r(-psi / I.psi_inf);
+        const R lg = log1p_eos(-psi / I.psi_inf);
         sigma = I.sigma0 * (R(1) + I.E0 * lg);
         mcoef = I.sigma0 * I.E0 / (I.psi_inf - psi);
         return true;
