@@ -54,7 +54,7 @@ constexpr int kSolveMaxBlocks = 256;  // blocks of a gang at most
 // surfactant sum of the tile
 struct __align__(16) SolveRec {
     float m[8];
-    float sum[4];  // of the two rounds: hi, hi, lo, lo
+    double2 sum;  // of the two rounds
 };
 constexpr size_t kSolveRecBytes = 2 * (size_t)kSolveMaxBlocks * sizeof(SolveRec);
 
@@ -149,19 +149,24 @@ __device__ __forceinline__ void lane_sums(float2 &hi, float2 &lo, int o) {
 // a plane's element at a byte offset (32 bits: one register an address)
 __device__ __forceinline__ float &at(float *p, unsigned o) { return *(float *)((char *)p + o); }
 
+// d <= tol x, the product not rounded (as in double precision)
+__device__ __forceinline__ bool at_most(float d, float tol, float x) {
+    const float p = __fmul_rn(tol, x);
+    return d < p || (d == p && !(fmaf(tol, x, -p) < 0.f));
+}
 // the decision of round_converged from the maxima themselves (m: |d psi|,
 // |d C|, |psi|, |C|; before: the largest update of the round before)
 __device__ __forceinline__ bool solve_converged(const float *m, float before, bool first,
                                                 float tol) {
-    const float p = tol * m[2], c = tol * m[3];
-    if (m[0] <= p && m[1] <= c) return true;
-    if (first || !(m[0] <= 8.f * p && m[1] <= 8.f * c)) return false;
+    if (at_most(m[0], tol, m[2]) && at_most(m[1], tol, m[3])) return true;
+    if (first || !(at_most(m[0], 8.f * tol, m[2]) && at_most(m[1], 8.f * tol, m[3]))) return false;
     return fmaxf(m[0], m[1]) >= 0.5f * before;
 }
 
 // tile (bx, by), block `blk` of the nb of grid I's gang.  FP64 runs at 1/64 of
-// FP32's rate and its chains are long here, so sums are compensated FP32 pairs,
-// exact to about 48 bits, up to the total.  The code is kept short (loops over
+// FP32's rate, so the surfactant is summed in compensated FP32 pairs within a
+// warp (256 cells; exact to about 48 bits) and in FP64 across warps and blocks,
+// the latter once, when the round that ends the solve is known.  The code is kept short (loops over
 // a thread's cells are rolled where the cells can pass through shared memory): with
 // little work a thread, the time of a launch is that of fetching its
 // instructions; unrolled over the eight cells it had 144 KB of code and took
@@ -179,10 +184,12 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
     float2 *Fr = Xs;
     float2 *Sn = (float2 *)(smem + 2 * S::w_bytes + S::x_bytes);
     __shared__ __align__(16) float redm[NW][8], redb[8][8];
-    __shared__ float4 reds[NW];  // sums of two rounds (hi, hi, lo, lo)
+    __shared__ float4 reds[NW];  // a warp's sums of two rounds (hi, hi, lo, lo)
+    __shared__ double2 sums[kSolveMaxBlocks];  // the blocks' sums of the last phase
     __shared__ struct {
-        float m0h, m0l;  // the conserved total as an FP32 pair
-        int ok;          // the barrier's wait ended well
+        double M0;     // the conserved total
+        float dscale;  // rescale step
+        int ok;        // the barrier's wait ended well
     } st;
     __shared__ uint4 offs[kSolveThreads];
     const int tid = threadIdx.x, l = tid & 31, w = tid >> 5;
@@ -392,19 +399,14 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
     put(0);
     put(1);
     const bool live = 4 * w < RY;  // (the warp has rows of the region)
-    if (tid == 0) {
-        const double M0 = ctl->M0;
-        const float h = float(M0);
-        st.m0h = h;
-        st.m0l = float(M0 - double(h));
-    }
+    if (tid == 0) st.M0 = ctl->M0;
     __syncthreads();
 
     // 4. phases of NR rounds
     const float2 om = make_float2(I.omega, I.omega);
     int rounds = 0;
     bool conv = false, keep = false;       // keep: the result is the kept round's
-    float before = 0.f, th = 0.f, tl = 0.f;  // the round's largest update, its total
+    float before = 0.f;                    // the round's largest update
     unsigned int bt = 0;
 #pragma unroll 1
     for (int ph = 0;; ph++) {
@@ -552,10 +554,15 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
             v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
             v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 16));
             const float4 u = reds[l & (NW - 1)];
-            float2 hi = make_float2(u.x, u.y), lo = make_float2(u.z, u.w);
-            lane_sums(hi, lo, NW / 2);
+            double2 s = make_double2(double(u.x) + double(u.z), 0.0);
+            if (NR > 1) s.y = double(u.y) + double(u.w);
+#pragma unroll
+            for (int o = NW / 2; o > 0; o >>= 1) {
+                s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+                if (NR > 1) s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+            }
             if (l < 8) recs[blk].m[l] = v;
-            if (l == 0) *(float4 *)recs[blk].sum = make_float4(hi.x, hi.y, lo.x, lo.y);
+            if (l == 0) recs[blk].sum = s;
             __syncwarp();
             if (l == 0) {
                 // (release: the block's writes before its last barrier, and the
@@ -587,20 +594,18 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
                 if (has(IN, r, 1)) X[r][1] = make_float2(p.y, c.y);
             }
         if (32 * w < nb) {
-            float4 v[NR], u = make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 v[NR];
 #pragma unroll
             for (int n = 0; n < NR; n++)
-                v[n] = tid < nb ? __ldcg((const float4 *)&recs[tid].m[4 * n]) : u;
-            if (tid < nb) u = __ldcg((const float4 *)recs[tid].sum);
-            float2 hi = make_float2(u.x, u.y), lo = make_float2(u.z, u.w);
+                v[n] = tid < nb ? __ldcg((const float4 *)&recs[tid].m[4 * n])
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (tid < nb) sums[tid] = __ldcg(&recs[tid].sum);
 #pragma unroll
             for (int n = 0; n < NR; n++) {
                 v[n] = make_float4(warp_max_pos(v[n].x), warp_max_pos(v[n].y), warp_max_pos(v[n].z),
                                    warp_max_pos(v[n].w));
                 if (l == 0) *(float4 *)&redb[w][4 * n] = v[n];
             }
-            lane_sums(hi, lo, 16);
-            if (l == 0) reds[w] = make_float4(hi.x, hi.y, lo.x, lo.y);
         }
         put(0);
         __syncthreads();
@@ -610,17 +615,13 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
         for (int n = 0; n < NR; n++)
             if (!stop) {
                 float mm[4] = {0.f, 0.f, 0.f, 0.f};
-                th = tl = 0.f;
 #pragma unroll 1
                 for (int j = 0; 32 * j < nb; j++) {
-                    const float4 v = *(const float4 *)&redb[j][4 * n], u = reds[j];
+                    const float4 v = *(const float4 *)&redb[j][4 * n];
                     mm[0] = fmaxf(mm[0], v.x);
                     mm[1] = fmaxf(mm[1], v.y);
                     mm[2] = fmaxf(mm[2], v.z);
                     mm[3] = fmaxf(mm[3], v.w);
-                    float e;
-                    th = two_sum(th, n ? u.y : u.x, e);
-                    tl = (tl + (n ? u.w : u.z)) + e;
                 }
                 conv = solve_converged(mm, before, rounds == 0, I.sor_tol);
                 before = fmaxf(mm[0], mm[1]);
@@ -630,10 +631,8 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
             }
         if (stop) break;
     }
-    // 5. rescale: x (1 + d), d = s - 1, rounded without bias (rescale_one)
-    float e;
-    const float d = two_sum(st.m0h, -th, e), t = th + tl;  // (s = M0 / total)
-    const float dscale_f = t > 0.f ? fdiv(d + (e + (st.m0l - tl)), t) : 0.f;
+    // 5. the round's total, and the rescale: x (1 + d), d = M0 / total - 1,
+    //    rounded without bias (rescale_one)
     const float2 *res = keep ? Sn : Xs;
     __syncthreads();  // (the halo's copies in Xs have been written)
     if (!keep)
@@ -641,6 +640,19 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
         for (int r = 0; r < 4; r++)
 #pragma unroll
             for (int q = 0; q < 2; q++) Xs[slot(r, q)] = X[r][q];
+    double total = 0.0, scale = 1.0;
+    if (w == 0) {
+        const bool second = NR > 1 && !keep;
+        for (int k = l; k < nb; k += 32) total += second ? sums[k].y : sums[k].x;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+        if (l == 0) {
+            if (total > 0) scale = st.M0 / total;
+            st.dscale = float(scale - 1.0);
+        }
+    }
+    __syncthreads();
+    const float dscale_f = st.dscale;
 #pragma unroll 1
     for (int k = 0; k < 8; k++) {
         if (!((mask >> (OWN + k)) & 1)) continue;
@@ -651,8 +663,6 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
         at(I.C, 4u * c) = rescale_one(v.y, 0.0, dscale_f, rescale_key(c, 1, step0));
     }
     if (blk != 0 || tid != 0) return;
-    const double total = double(th) + double(tl);
-    const double scale = total > 0 ? ctl->M0 / total : 1.0;
     ctl->pre = total;
     ctl->scale = scale;
     ctl->dscale = scale - 1.0;

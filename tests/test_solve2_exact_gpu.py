@@ -1,0 +1,60 @@
+"""The resident solve (k_solve2; kb_solve2 of a batch) against the launches of
+one round each: the same total, the same rescale, the same stop.
+
+Both sum exact products in compensated FP32 strips and the strips in FP64.  The
+strips' errors (2^-48 of a strip) average out over 10^3 and more of them, and an
+FP64 sum of some 20 levels is off by 2^-53 times about their root: two ulps of
+the total (2^-52 of it each) and one to spare.  Sums of FP32 pairs up to the grid
+are off by 4 to 8."""
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+TOTAL_TOL = 3 * 2.0 ** -52
+
+
+def solver(cfg, f, storage, on, variant=0):
+    from paper_2311_15242_gb300 import Solver
+    s = Solver(cfg, storage=storage)
+    s.set_sor_tile(variant)
+    s.set_sor_persistent(on)
+    s.init_fields(f["phi"], f["psi"], f["C"], f["u"])
+    return s
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("n,variant", [(128, 0), (251, 0), (400, 0), (400, 5), (500, 0), (600, 0)])
+def test_total_is_summed_in_double_precision(n, variant, storage):
+    """One step: the solves' inputs are the same, and so are psi and C but for
+    cells that hold less than 1e-14 of the largest value."""
+    cfg = W.droplet_adsorption_2d(n=n, R=n * 0.2)
+    f = W.initial_fields(cfg, seed=5, noise=0.02, u0=1e-3)
+    pre = []
+    for on in (True, False):
+        s = solver(cfg, f, storage, on, variant)
+        s.step(1)
+        pre.append(s.step_result()[1])
+        s.close()
+    assert abs(pre[0] / pre[1] - 1.0) <= TOTAL_TOL, pre
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+def test_totals_of_a_batch_of_several_waves(storage):
+    """Nine instances (more than one wave of tiles) against their own contexts
+    with a launch a round."""
+    from paper_2311_15242_gb300 import Batch
+    cfgs = [W.droplet_adsorption_2d(n=200 + 24 * k, R=40.0 + 4 * k) for k in range(9)]
+    fs = [W.initial_fields(c, seed=k, noise=0.02, u0=1e-3) for k, c in enumerate(cfgs)]
+    b = Batch(cfgs, storage=storage)
+    for k, f in enumerate(fs):
+        b.init_fields(k, f["phi"], f["psi"], f["C"], f["u"])
+    b.step(1)
+    d = b.diagnostics()
+    b.close()
+    for k, (c, f) in enumerate(zip(cfgs, fs)):
+        s = solver(c, f, storage, False)
+        s.step(1)
+        assert abs(d[k]["surf_pre_rescale"] / s.step_result()[1] - 1.0) <= TOTAL_TOL, k
+        s.close()
