@@ -292,11 +292,12 @@ int lbs_set_sor_tile(lbs_ctx *c, int variant);
  * LBS_EINVAL (no context), LBS_ECUDA. */
 int lbs_set_sor_persistent(lbs_ctx *c, int on);
 
-/* The most polls (about 64 ns each) a block of the one-launch SOR waits at
- * the grid barrier between rounds before it gives up: the step then reports
+/* The most polls (about 64 ns each) a block of a one-launch solve (2D, or 3D
+ * sweeps) waits at a grid barrier before it gives up: the step then reports
  * LBS_ETIMEOUT (at the next lbs_sync or lbs_diagnostics) instead of waiting
- * on.  Default 2^24, about a second; 0 gives up at once unless every block
- * has arrived.  After a timeout the fields of that step are not valid
+ * on.  Default 2^24, about a second; below 3 (the time of one look at the
+ * arrivals, about 0.2 us) a block gives up at once unless it is the last to
+ * arrive.  After a timeout the fields of that step are not valid
  * (initialise them again or load a saved state); the next step's launch
  * starts with a clear barrier.  Errors: LBS_EINVAL (no context, negative limit), LBS_ECUDA. */
 int lbs_set_sor_wait_limit(lbs_ctx *c, long long polls);
@@ -387,11 +388,18 @@ int lbs_batch_diagnostics(lbs_batch *b, lbs_diag *d);
  * launches with a host-driven SOR loop (for kernel profilers). */
 int lbs_batch_set_graph(lbs_batch *b, int enable);
 
+/* As lbs_set_sor_wait_limit, for the one launch that solves all instances:
+ * the instances whose blocks gave up report LBS_ETIMEOUT (lbs_batch_status),
+ * and their fields are not valid until they are initialised again.  A solve
+ * takes at most about a millisecond, and a block waits for others no longer
+ * than the instances before its own take. */
+int lbs_batch_set_sor_wait_limit(lbs_batch *b, long long polls);
+
 /* Kernel launches of one batch step (SOR rounds as of the last diagnostics). */
 int lbs_batch_step_kernel_count(const lbs_batch *b);
 
 /* Status of every instance since the last call, status[0..n-1] (lbs_status
- * codes: LBS_EDIVERGED, LBS_ENOCONV, ...), then cleared.  An instance whose
+ * codes: LBS_EDIVERGED, LBS_ENOCONV, LBS_ETIMEOUT, ...), then cleared.  An instance whose
  * total surfactant went non-finite is skipped by every later step (its
  * state is frozen); the others go on.  lbs_batch_sync and
  * lbs_batch_get_fields do not clear these codes; lbs_batch_diagnostics

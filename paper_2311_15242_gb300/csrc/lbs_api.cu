@@ -474,8 +474,8 @@ struct Solver : Base {
         at[0].val.cooperative = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        long long polls = coop_polls;
-        void *args[] = {(void *)&I, (void *)&fsg, (void *)&maxr, (void *)&polls};
+        long long looks = barrier_looks(coop_polls);
+        void *args[] = {(void *)&I, (void *)&fsg, (void *)&maxr, (void *)&looks};
         CK(cudaLaunchKernelExC(&cfg, L3::fs_fn(), args));
         return LBS_OK;
     }
@@ -547,16 +547,16 @@ struct Solver : Base {
         at[0].val.cooperative = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        long long polls = coop_polls;
+        long long looks = barrier_looks(coop_polls);
         if (solve_ok) {
             cfg.gridDim = dim3(sg.ntx * sg.nty, 1, 1);
             cfg.blockDim = dim3(kSolveThreads, 1, 1);
             cfg.dynamicSmemBytes = sf.smem;
-            void *args[] = {(void *)&I, (void *)&sg, (void *)&maxr, (void *)&polls};
+            void *args[] = {(void *)&I, (void *)&sg, (void *)&maxr, (void *)&looks};
             CK(cudaLaunchKernelExC(&cfg, sf.fn, args));
             return LBS_OK;
         }
-        void *args[] = {(void *)&I, (void *)&maxr, (void *)&polls};
+        void *args[] = {(void *)&I, (void *)&maxr, (void *)&looks};
         CK(cudaLaunchKernelExC(&cfg, sor2_coop_kernel<R>(s2), args));
         return LBS_OK;
     }

@@ -213,14 +213,14 @@ struct GangItem {
 template <int K, int NR>
 __global__ void __launch_bounds__(kSolveThreads, 1)
     kb_solve2(const Inst<float> *__restrict__ insts, const GangItem *__restrict__ items, int waves,
-              int max_rounds, long long max_polls) {
+              int max_rounds, long long max_looks) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Inst<float> sI;
     int cur = -1, alive = 0;
     for (int k = 0; k < waves; k++) {
         const GangItem it = items[(size_t)k * gridDim.x + blockIdx.x];
         if (it.inst < 0 || !load_inst(insts, it.inst, sI, cur, alive)) continue;
-        solve2_tile<K, NR>(sI, it.g, it.bx, it.by, it.blk, it.nb, max_rounds, max_polls, smem_raw);
+        solve2_tile<K, NR>(sI, it.g, it.bx, it.by, it.blk, it.nb, max_rounds, max_looks, smem_raw);
     }
 }
 
@@ -277,6 +277,7 @@ struct lbs_batch {
     virtual int set_graph(int on) = 0;
     virtual int status(int *st) = 0;
     virtual int set_active(int k, int on) = 0;
+    virtual int set_sor_wait_limit(long long polls) = 0;
     char err[512] = {0};
 };
 
@@ -332,6 +333,7 @@ struct Batch : lbs_batch {
         int waves, blocks;
     } gang = {};
     GangItem *d_gang = nullptr;
+    long long polls = kBarrierPolls;  // wait limit of kb_solve2's barriers
     int n_cells = 0, n_sor = 0, n_surf = 0;
     int tx = 32, ty = 8, sv = 0;
     int g_cells[NOPS] = {0}, g_sor = 0, g_surf = 0;
@@ -691,9 +693,9 @@ struct Batch : lbs_batch {
             at[0].val.cooperative = 1;
             cfg.attrs = at;
             cfg.numAttrs = 1;
-            long long polls = kBarrierPolls;
+            long long looks = barrier_looks(polls);
             void *args[] = {(void *)&d_insts, (void *)&d_gang, (void *)&gang.waves,
-                            (void *)&max_rounds, (void *)&polls};
+                            (void *)&max_rounds, (void *)&looks};
             BCK(cudaLaunchKernelExC(&cfg, gang.fn, args));
             return LBS_OK;
         }
@@ -889,6 +891,17 @@ struct Batch : lbs_batch {
         return (kFused ? live : 3) + (gang.fn ? 1 : 4 + last_rounds);
     }
 
+    int set_sor_wait_limit(long long p) override {
+        if (p < 0) {
+            berr(this, "wait limit must be >= 0 polls");
+            return LBS_EINVAL;
+        }
+        BCK(cudaStreamSynchronize(stream));
+        drop_graphs();
+        polls = p;
+        return LBS_OK;
+    }
+
     int set_graph(int on) override {
         use_graph = bool(on);
         return LBS_OK;
@@ -988,6 +1001,11 @@ int lbs_batch_diagnostics(lbs_batch *b, lbs_diag *d) {
 int lbs_batch_set_graph(lbs_batch *b, int enable) {
     if (!b) return LBS_EINVAL;
     return b->set_graph(enable);
+}
+
+int lbs_batch_set_sor_wait_limit(lbs_batch *b, long long polls) {
+    if (!b) return LBS_EINVAL;
+    return b->set_sor_wait_limit(polls);
 }
 
 int lbs_batch_step_kernel_count(const lbs_batch *b) { return b ? b->kernel_count() : 0; }

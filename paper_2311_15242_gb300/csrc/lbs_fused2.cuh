@@ -682,10 +682,10 @@ __global__ void k_grad2n(Inst<R> I) {
 //      the partials of the last round, added by every block in the same
 //      order;
 //   4. rescale psi, C by M0 / total (Sec. 2.2) into the canonical buffers.
-// Every barrier waits at most max_polls polls, then reports ST_TIMEOUT.
+// Every barrier looks at the arrivals at most max_looks times, then reports ST_TIMEOUT.
 // ---------------------------------------------------------------------------
 template <typename R, int TX, int TY, int K, int BS>
-__global__ void __launch_bounds__(BS) k_sorfuse2(Inst<R> I, int max_rounds, long long max_polls) {
+__global__ void __launch_bounds__(BS) k_sorfuse2(Inst<R> I, int max_rounds, long long max_looks) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const unsigned int nb = gridDim.x;
     const int tid = threadIdx.x;
@@ -709,7 +709,7 @@ __global__ void __launch_bounds__(BS) k_sorfuse2(Inst<R> I, int max_rounds, long
             y++;
         }
     }
-    if (!grid_barrier(ctl, nb, bt, max_polls)) return;
+    if (!grid_barrier(ctl, nb, bt, max_looks)) return;
     // 2. SOR rounds.  As a block stores its tiles' cells it also sums their
     //    surfactant; the round that ends the solve thus leaves the block
     //    partials of the total in I.part (3) with no pass of its own.
@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(BS) k_sorfuse2(Inst<R> I, int max_rounds, long
             double bsum[1];
             block_sum<BS, 1>(v, bsum);
             if (tid == 0) I.part[blockIdx.x] = bsum[0];
-            if (!grid_barrier(ctl, nb, bt, max_polls)) return;
+            if (!grid_barrier(ctl, nb, bt, max_looks)) return;
             conv = round_converged<R>(ctl, round, double(I.sor_tol));
             if (conv || round + 1 >= max_rounds) break;
         }
@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(BS) k_sorfuse2(Inst<R> I, int max_rounds, long
         double bsum[1];
         block_sum<BS, 1>(v, bsum);
         if (tid == 0) I.part[blockIdx.x] = bsum[0];
-        if (!grid_barrier(ctl, nb, bt, max_polls)) return;
+        if (!grid_barrier(ctl, nb, bt, max_looks)) return;
     }
     // every block adds the block partials in the same order
     double acc[1] = {0.0};

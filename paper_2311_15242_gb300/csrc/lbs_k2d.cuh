@@ -1302,10 +1302,31 @@ __device__ __forceinline__ void sor_tile2(const Inst<R> &I, int round, int bx, i
 // ---------------------------------------------------------------------------
 // Grid barrier of the one-launch SOR (k_sorfuse2, lbs_fused2.cuh): every
 // block of a cooperative launch arrives, the last one releases the others.
-// A barrier waits at most max_polls polls (the default, kBarrierPolls, is
-// about a second), then reports ST_TIMEOUT and returns false.
+// A barrier looks at the counter at most max_looks times, then reports
+// ST_TIMEOUT and returns false.
 // ---------------------------------------------------------------------------
+// the wait limit in polls of 64 ns (the default is about a second), and in looks:
+// one takes 170 ns (a load through L2), 207 with the pause of grid_barrier (1 to
+// 152 blocks waiting).  A limit below that leaves no time for one: only the block
+// that arrives last goes on.
 constexpr long long kBarrierPolls = 1LL << 24;
+constexpr long long barrier_looks(long long polls) { return polls / 3; }
+
+// one arrival (release: the thread's writes and those it has seen by a block
+// barrier before); where the limit leaves no look at the counter, whether it
+// was the last one, else true
+__device__ __forceinline__ bool barrier_arrive(Ctl *ctl, unsigned int target, long long max_looks) {
+    if (max_looks > 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctl->bar_count) : "memory");
+        return true;
+    }
+    unsigned int before;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;"
+                 : "=r"(before)
+                 : "l"(&ctl->bar_count)
+                 : "memory");
+    return before + 1 >= target;
+}
 
 // Grid barrier of a cooperative launch: every block adds one arrival to a
 // counter that the kernel before the launch cleared, and waits until the
@@ -1316,24 +1337,21 @@ constexpr long long kBarrierPolls = 1LL << 24;
 // short of every later target, so the launch's later barriers give up too,
 // and the next launch starts from a cleared counter).
 __device__ __forceinline__ bool grid_barrier(Ctl *ctl, unsigned int nblocks,
-                                             unsigned int &target, long long max_polls) {
+                                             unsigned int &target, long long max_looks) {
     __shared__ int ok;
     target += nblocks;
     __syncthreads();
     if (threadIdx.x == 0) {
-        ok = 1;
         __threadfence();
-        atomicAdd(&ctl->bar_count, 1u);
+        ok = barrier_arrive(ctl, target, max_looks);
         const volatile unsigned int *count = &ctl->bar_count;
-        long long polls = 0;
-        while (*count < target) {
-            if (++polls > max_polls) {
+        for (long long looks = 0; ok && *count < target;) {
+            if (++looks > max_looks)
                 ok = 0;
-                atomicOr(&ctl->status, int(ST_TIMEOUT));
-                break;
-            }
-            __nanosleep(32);
+            else
+                __nanosleep(32);
         }
+        if (!ok) atomicOr(&ctl->status, int(ST_TIMEOUT));
         __threadfence();
     }
     __syncthreads();

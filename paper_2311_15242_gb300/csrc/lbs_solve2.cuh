@@ -174,7 +174,7 @@ __device__ __forceinline__ bool solve_converged(const float *m, float before, bo
 template <int K, int NR>
 __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeom &g, int bx,
                                             int by, int blk, int nb, int max_rounds,
-                                            long long max_polls, unsigned char *smem) {
+                                            long long max_looks, unsigned char *smem) {
     constexpr int N = kSolveRegion, H = 2 * K * NR, NW = kSolveThreads / 32;
     using S = SolveSmem<NR>;
     constexpr int FS = S::FS;
@@ -567,16 +567,11 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
             if (l == 0) {
                 // (release: the block's writes before its last barrier, and the
                 // record.  Relaxed polls: an acquire empties the L1 every time)
-                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctl->bar_count)
-                             : "memory");
+                int ok = barrier_arrive(ctl, bt, max_looks);
                 const volatile unsigned int *count = &ctl->bar_count;
-                int ok = 1;
-                for (long long polls = 0; *count < bt;)
-                    if (++polls > max_polls) {
-                        ok = 0;
-                        atomicOr(&ctl->status, int(ST_TIMEOUT));
-                        break;
-                    }
+                for (long long looks = 0; ok && *count < bt;)
+                    if (++looks > max_looks) ok = 0;
+                if (!ok) atomicOr(&ctl->status, int(ST_TIMEOUT));
                 __threadfence();
                 st.ok = ok;
             }
@@ -667,9 +662,10 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
     ctl->scale = scale;
     ctl->dscale = scale - 1.0;
     ctl->dscale_f = dscale_f;
-    if (!conv) ctl->status |= ST_NOCONV;
+    // (atomic: another block may be giving up its wait)
+    if (!conv) atomicOr(&ctl->status, int(ST_NOCONV));
     if (!isfinite(total)) {
-        ctl->status |= ST_DIVERGED;
+        atomicOr(&ctl->status, int(ST_DIVERGED));
         ctl->dead = 1;
     }
     ctl->sor_iters = rounds * K;
@@ -680,10 +676,10 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
 
 template <int K, int NR>
 __global__ void __launch_bounds__(kSolveThreads, 1)
-    k_solve2(Inst<float> I, SolveGeom g, int max_rounds, long long max_polls) {
+    k_solve2(Inst<float> I, SolveGeom g, int max_rounds, long long max_looks) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     solve2_tile<K, NR>(I, g, blockIdx.x % g.ntx, blockIdx.x / g.ntx, blockIdx.x, gridDim.x,
-                       max_rounds, max_polls, smem_raw);
+                       max_rounds, max_looks, smem_raw);
 }
 
 }  // namespace lbs

@@ -64,7 +64,7 @@ inline bool sor3_geom(int nx, int ny, int nz, const int *wall, int blocks, Sor3G
 }
 
 __global__ void __launch_bounds__(kSor3Threads, 1)
-    k_sor_fs3(Inst<float> I, Sor3Geom g, int max_rounds, long long max_polls) {
+    k_sor_fs3(Inst<float> I, Sor3Geom g, int max_rounds, long long max_looks) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *Xs = (float2 *)smem_raw;                  // [slot][row][q][lane]
     float2 *Ws = Xs + 4 * kSor3Rows * 64;
@@ -308,12 +308,13 @@ __global__ void __launch_bounds__(kSor3Threads, 1)
             atomic_max_pos(&ctl->sweep[round][tid], double(m));
             __threadfence();  // (before the arrival that the next barrier makes)
         }
-        if (!grid_barrier(ctl, gridDim.x, bt, max_polls)) return;
+        if (!grid_barrier(ctl, gridDim.x, bt, max_looks)) return;
         if (tid == 0) {
             const bool conv = round_converged<float>(ctl, round, double(I.sor_tol));
             s_stop = conv || round + 1 >= max_rounds;
             if (blockIdx.x == 0 && s_stop) {
-                if (!conv) ctl->status |= ST_NOCONV;
+                // (atomic: another block may be giving up its wait)
+                if (!conv) atomicOr(&ctl->status, int(ST_NOCONV));
                 ctl->sor_exec = round + 1;
             }
         }

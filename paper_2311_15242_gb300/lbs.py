@@ -28,6 +28,7 @@ EXPORTS = ("lbs_params_default", "lbs_workspace_bytes", "lbs_create",
            "lbs_batch_init_fields", "lbs_batch_set_tiles", "lbs_batch_step", "lbs_batch_sync",
            "lbs_batch_get_fields", "lbs_batch_diagnostics", "lbs_batch_set_graph",
            "lbs_batch_step_kernel_count", "lbs_batch_status", "lbs_batch_set_active",
+           "lbs_batch_set_sor_wait_limit",
            "lbs_batch_destroy", "lbs_batch_last_error",
            "lbs_mlp_create", "lbs_mlp_param_count", "lbs_mlp_init", "lbs_mlp_set_params",
            "lbs_mlp_get_params", "lbs_mlp_forward", "lbs_mlp_gradient", "lbs_mlp_set_grad",
@@ -129,6 +130,7 @@ def load(build_if_missing: bool = True):
     L.lbs_batch_get_fields.argtypes = [C.c_void_p, C.c_int, _DP, _DP, _DP, _DP, _DP]
     L.lbs_batch_diagnostics.argtypes = [C.c_void_p, C.POINTER(LbsDiag)]
     L.lbs_batch_set_graph.argtypes = [C.c_void_p, C.c_int]
+    L.lbs_batch_set_sor_wait_limit.argtypes = [C.c_void_p, C.c_longlong]
     L.lbs_batch_step_kernel_count.argtypes = [C.c_void_p]
     L.lbs_batch_status.argtypes = [C.c_void_p, C.POINTER(C.c_int)]
     _FP = C.POINTER(C.c_float)
@@ -392,6 +394,11 @@ class Batch:
 
     def set_graph(self, on=True):
         self._check(self.L.lbs_batch_set_graph(self.h, int(bool(on))))
+
+    def set_sor_wait_limit(self, polls):
+        """Most polls a block waits at the grid barriers of the one launch that
+        solves all instances (see lbs_batch_set_sor_wait_limit)."""
+        self._check(self.L.lbs_batch_set_sor_wait_limit(self.h, int(polls)))
 
     def step(self, n=1):
         self._check(self.L.lbs_batch_step(self.h, int(n)))
