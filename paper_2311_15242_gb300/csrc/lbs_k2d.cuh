@@ -240,6 +240,16 @@ template <typename R>
 __device__ __forceinline__ R frac(const Inst<R> &I, long long j, bool red) {
     return frac_of(I, I.rhoR, I.rhoB, j, red);
 }
+// chi = 1 - rho^N, twice the blue fraction.  The sum of the fractions' parts is
+// rounded once, here and in every kernel that forms chi: the solve's forms
+// agree to the bit only if their weights do.
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+template <typename R>
+__device__ __forceinline__ R chi_of(const Inst<R> &I, R rR, R rB) {
+    const R xb = rB * I.inv_rhoB0;
+    return R(2) * fdiv(xb, fma_rn(rR, I.inv_rhoR0, xb));
+}
 
 // gradient and weights of cell (x, y) from the colour densities rR, rB and
 // colour function rN (the current moments, or the next ones of the fused step)
@@ -264,7 +274,7 @@ __device__ __forceinline__ void grad2_cell_from(const Inst<R> &I, int x, int y, 
     I.gx[c] = gx;
     I.gy[c] = gy;
     I.a[c] = sqrt(gx * gx + gy * gy);
-    I.chi[c] = R(2) * frac_of(I, rR, rB, c, false);
+    I.chi[c] = chi_of(I, rR[c], rB[c]);
 }
 
 template <typename R>

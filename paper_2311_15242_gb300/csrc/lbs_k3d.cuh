@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(256) k_grad3(Inst<R> I, int guess = 1) {
         I.gy[c] = gy;
         I.gz[c] = gz;
         I.a[c] = sqrt(gx * gx + gy * gy + gz * gz);
-        I.chi[c] = R(2) * fr[0][q];
+        I.chi[c] = chi_of(I, I.rhoR[c], I.rhoB[c]);
         if (guess) sor_guess(I, c);
     }
 }

@@ -10,9 +10,11 @@
 // holds the cell pairs 2 l, 2 l + 1 of the rows 4 w .. 4 w + 3: psi, C, and the
 // faces and inverse diagonals of their rows (the right-hand sides wait in shared
 // memory for want of registers).  An update is that of sor_tile2_cb, operation by
-// operation, so the results are its own to the bit but for the rounding of
-// the rescale factor.  The x-neighbour outside the pair comes from the adjacent lane by shuffle; of the y-neighbours only
-// those in another warp's rows go through shared memory.  A half-sweep
+// operation and rounding by rounding, so the results are its own to the bit
+// (but where the totals, summed in other orders, round the rescale step apart:
+// some four steps in a million).  The x-neighbour outside the pair comes from the
+// adjacent lane by shuffle; of the y-neighbours only those in another warp's rows
+// go through shared memory.  A half-sweep
 // updates one cell of every pair, spreads the error of the stale region edge
 // by one cell, and ends with a block barrier.
 //
@@ -31,6 +33,8 @@
 // 4.4 for 4 sweeps, 2 x 5 from publishing the tile to the decision); at 64 x 517
 // (33 blocks, 6 sweeps) 53 -> 33 us, at 241 x 1011 (odd periodic axis) 90 -> 41.
 #pragma once
+
+#include <type_traits>
 
 #include "lbs_k2d.cuh"
 
@@ -295,6 +299,13 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
         b[r][0] = make_float2(u.x, v.x);
         b[r][1] = make_float2(u.y, v.y);
     }
+    // (chi waits in the weights' place until they are formed; behind the loads
+    // above, not before them: 0.9 us less at 256 x 1024)
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        Ws[slot(r, 0)].y = chi_of(I, rR[r].x, rB[r].x);
+        Ws[slot(r, 1)].y = chi_of(I, rR[r].y, rB[r].y);
+    }
     const bool seam = __syncthreads_or(mask >> FLIP) != 0;  // (of an odd periodic y axis)
     // 2. gradient and weights of t+1 (grad2_cell_from): the tile's go to the
     //    planes that the next step and the exports read
@@ -320,7 +331,7 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
             gx[q] *= c;
             gy[q] *= c;
             a[q] = sqrt(gx[q] * gx[q] + gy[q] * gy[q]);
-            chi[q] = 2.f * f[q * FS].y;
+            chi[q] = Ws[slot(r, q)].y;
             Ws[slot(r, q)] = make_float2(a[q] + I.eps_w, chi[q] + I.eps_w);
         }
         // (a tile's cells are grid cells: no mapping)
@@ -403,7 +414,6 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
     __syncthreads();
 
     // 4. phases of NR rounds
-    const float2 om = make_float2(I.omega, I.omega);
     int rounds = 0;
     bool conv = false, keep = false;       // keep: the result is the kept round's
     float before = 0.f;                    // the round's largest update
@@ -416,15 +426,18 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
             float2 md = make_float2(0.f, 0.f), mx = make_float2(0.f, 0.f);
             auto fold = [&](float2 d, float2 x, bool mine) {
                 if (mine) {
-                    md.x = fmaxf(md.x, fabsf(om.x * d.x));
-                    md.y = fmaxf(md.y, fabsf(om.y * d.y));
-                    mx.x = fmaxf(mx.x, fabsf(fmaf(om.x, d.x, x.x)));
-                    mx.y = fmaxf(mx.y, fabsf(fmaf(om.y, d.y, x.y)));
+                    md.x = fmaxf(md.x, fabsf(d.x));
+                    md.y = fmaxf(md.y, fabsf(d.y));
+                    mx.x = fmaxf(mx.x, fabsf(x.x));
+                    mx.y = fmaxf(mx.y, fabsf(x.y));
                 }
             };
-#pragma unroll 1
-            for (int k = 0; k < K; k++) {
-                const bool count = k == K - 1;  // (the last sweep's updates count)
+            // (the last sweep's updates count, and it rounds them before it adds
+            // them, which the others do not: sor_tile2_cb's roundings.  Two bodies:
+            // one with the choice inside takes 0.3 us more at 64 x 517, 0.9 at 256
+            // x 1024)
+            auto sweep = [&](auto last) {
+                constexpr bool LAST = decltype(last)::value;
                 auto update = [&](int r, int q, float2 side, float2 xso, float2 xno) {
                     float2 x = fma2(fE[r][q], q ? side : X[r][1], Bs[slot(r, q)]);
                     x = fma2(fN[r][q], xno, x);
@@ -432,8 +445,13 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
                     x = fma2(r ? fN[r ? r - 1 : 0][q] : fS[q], xso, x);
                     const float2 o = X[r][q];
                     x = fma2(x, iv[r][q], make_float2(-o.x, -o.y));
-                    if (count) fold(x, o, has(OWN, r, q));
-                    X[r][q] = fma2(om, x, o);
+                    if (LAST) {
+                        const float2 d = make_float2(__fmul_rn(I.omega, x.x), __fmul_rn(I.omega, x.y));
+                        X[r][q] = make_float2(__fadd_rn(o.x, d.x), __fadd_rn(o.y, d.y));
+                        fold(d, X[r][q], has(OWN, r, q));
+                    } else {
+                        X[r][q] = make_float2(fmaf(I.omega, x.x, o.x), fmaf(I.omega, x.y, o.y));
+                    }
                 };
                 // half-sweep t reads copy t of the rows at the warps' edges (row
                 // 4 w - 1 is row 3 of the warp below, row 4 w + 4 row 0 of the one
@@ -499,7 +517,10 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
                         __syncthreads();
                     }
                 }
-            }
+            };
+#pragma unroll 1
+            for (int k = 0; k < K - 1; k++) sweep(std::false_type());
+            sweep(std::true_type());
             // the round's maxima and the surfactant of the tile: products exact
             // as hi + lo, sums compensated
             float2 hi = make_float2(0.f, 0.f), lo = make_float2(0.f, 0.f);

@@ -58,3 +58,29 @@ def test_totals_of_a_batch_of_several_waves(storage):
         s.step(1)
         assert abs(d[k]["surf_pre_rescale"] / s.step_result()[1] - 1.0) <= TOTAL_TOL, k
         s.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16"])
+@pytest.mark.parametrize("cfg,variant", [
+    (W.bubble_rise_2d(nx=64, ny=517, D_b=32.0, Eo=5.0, Bi=0.3), 0),    # odd periodic y
+    (W.bubble_rise_2d(nx=241, ny=300, D_b=64.0, Eo=10.0), 0),          # odd, walled x
+    (W.bubble_rise_2d(nx=256, ny=1024, D_b=64.0, Eo=10.0), 0),
+    (W.bubble_rise_2d(nx=128, ny=400, D_b=48.0, Eo=3.0), 3),           # 4 sweeps a round
+    (W.droplet_adsorption_2d(n=400, R=75.0), 0),                       # tails down to 1e-37
+    (W.droplet_adsorption_2d(n=63, R=15.0), 0),                        # odd: not resident
+], ids=["64x517", "241x300", "256x1024", "128x400-4", "droplet400", "droplet63"])
+def test_fields_equal_round_launches_to_the_bit(cfg, variant, storage):
+    """The same roundings in the weights and in every sweep.  Density ratio 10
+    (a factor 1 / rho^R0 whose product rounds) and FP16 populations, where
+    one different bit would send others after it."""
+    f = W.initial_fields(cfg, seed=5, noise=0.02, u0=1e-3)
+    s = [solver(cfg, f, storage, on, variant) for on in (True, False)]
+    for n in (1, 1, 10):
+        for q in s:
+            q.step(n)
+        a, b = s[0].fields(), s[1].fields()
+        assert {k: int((a[k] != b[k]).sum()) for k in a} == dict.fromkeys(a, 0)
+        a, b = s[0].macro(), s[1].macro()
+        assert {k: int((a[k] != b[k]).sum()) for k in a} == dict.fromkeys(a, 0)
+    for q in s:
+        q.close()
