@@ -119,7 +119,10 @@ __global__ void __launch_bounds__(kSor3Threads, 1)
                     }
                 }
             }
-            // a row's pair of a field on plane z (zeros outside the region or the grid)
+            // a row's pair of a field on plane z (zeros outside the region or the grid;
+            // the second cell of an odd row's last pair is padding, zero in psi and C
+            // since the state was initialised or loaded: faces have no weight
+            // towards it, but 0 times a NaN would be one)
             auto load2 = [&](const float *f, int z, int r) {
                 float2 v = make_float2(0.f, 0.f);
                 if (z >= 0 && has(in, r, 0)) v = *(const float2 *)((const char *)(f + z * plane) + off[r]);
