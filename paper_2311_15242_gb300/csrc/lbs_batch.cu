@@ -316,6 +316,7 @@ struct Batch : lbs_batch {
     int *d_act = nullptr;      // instance in the work lists (device copy of act)
     std::vector<int> act;      // host flags: instance in the work lists
     std::vector<int> st;       // sticky per-instance status (lbs_status codes)
+    std::vector<int> set;      // status words read back by collect
     WorkItem *d_cells = nullptr, *d_sor = nullptr, *d_surf = nullptr;
     // kb_fused2: its tile (16 x 8 or 32 x 16), the instances' descriptors, and
     // the streams of the launches beside the batch's own
@@ -334,6 +335,7 @@ struct Batch : lbs_batch {
     } gang = {};
     GangItem *d_gang = nullptr;
     long long polls = kBarrierPolls;  // wait limit of kb_solve2's barriers
+    bool ready = false;  // the work lists are those of the tiles and the active instances
     int n_cells = 0, n_sor = 0, n_surf = 0;
     int tx = 32, ty = 8, sv = 0;
     int g_cells[NOPS] = {0}, g_sor = 0, g_surf = 0;
@@ -434,6 +436,7 @@ struct Batch : lbs_batch {
         BCK(cudaMemset(d_bc, 0, sizeof(BatchCtl)));
         act.assign(n, 1);
         st.assign(n, 0);
+        set.assign(n, 0);
         BCK(cudaMalloc(&d_status, n * sizeof(int)));
         BCK(cudaMalloc(&d_act, n * sizeof(int)));
         BCK(cudaMemcpy(d_act, act.data(), n * sizeof(int), cudaMemcpyHostToDevice));
@@ -476,10 +479,12 @@ struct Batch : lbs_batch {
         fused_small = fused_tiles<32, 16>() <= sms / 2;
     }
     template <int TX, int TY>
-    void launch_fused(int k, cudaStream_t s) {
-        const Inst<R> &I = insts[k];
-        kb_fused2<R, P, TX, TY><<<dim3((I.nx + TX - 1) / TX, (I.ny + TY - 1) / TY), TX * TY,
-                                  Fuse2<R, TX, TY>::bytes(), s>>>(I);
+    cudaError_t launch_fused(int k, cudaStream_t s) {
+        Inst<R> &I = insts[k];
+        void *args[] = {(void *)&I};
+        return cudaLaunchKernel((void *)kb_fused2<R, P, TX, TY>,
+                                dim3((I.nx + TX - 1) / TX, (I.ny + TY - 1) / TY), dim3(TX * TY),
+                                args, Fuse2<R, TX, TY>::bytes(), s);
     }
     // the fused step of every active instance on s and the streams beside it
     int enqueue_fused(cudaStream_t s) {
@@ -490,19 +495,19 @@ struct Batch : lbs_batch {
             BCK(cudaEventRecord(fork, s));
             for (int i = 0; i < ns; i++) BCK(cudaStreamWaitEvent(side[i], fork, 0));
         }
-        for (int k = 0, at = 0; k < n; k++) {
+        cudaError_t e = cudaSuccess;
+        for (int k = 0, at = 0; k < n && e == cudaSuccess; k++) {
             if (!act[k]) continue;
             const int i = at++ % (ns + 1);
             cudaStream_t t = i ? side[i - 1] : s;
-            if (fused_small)
-                launch_fused<16, 8>(k, t);
-            else
-                launch_fused<32, 16>(k, t);
+            e = fused_small ? launch_fused<16, 8>(k, t) : launch_fused<32, 16>(k, t);
         }
+        // (joined also where a launch failed: a capture must not end forked)
         for (int i = 0; i < ns; i++) {
             BCK(cudaEventRecord(joined[i], side[i]));
             BCK(cudaStreamWaitEvent(s, joined[i], 0));
         }
+        BCK(e);
         return LBS_OK;
     }
 
@@ -615,6 +620,7 @@ struct Batch : lbs_batch {
         }
         BCK(cudaStreamSynchronize(stream));
         drop_graphs();
+        ready = false;
         tx = tx_;
         ty = ty_;
         sv = sv_;
@@ -656,7 +662,12 @@ struct Batch : lbs_batch {
             if (fk[o]) g_cells[o] = persistent_grid(fk[o], th, 0, n_cells);
         g_sor = persistent_grid(sor_kernel(sizeof(R) == 8, sv), sor_vbs(sv), sor_smem<R>(sv), n_sor);
         g_surf = persistent_grid((void *)kb_surf2<R, kSurfBS>, kSurfBS, 0, n_surf);
-        return set_gang();
+        int rg = set_gang();
+        if (rg) return rg;
+        // (the lists have arrived before work on the batch's stream)
+        BCK(cudaStreamSynchronize(0));
+        ready = true;
+        return LBS_OK;
     }
 
     int init(int k, const double *phi, const double *psi, const double *C,
@@ -764,6 +775,7 @@ struct Batch : lbs_batch {
         for (int k = 0; k < steps && !r; k++) r = enqueue_step(stream, true);
         cudaGraph_t out = nullptr;
         cudaError_t e = cudaStreamEndCapture(stream, &out);
+        if (r || e != cudaSuccess) drop_graphs();
         if (r) return r;
         if (e != cudaSuccess) {
             berr(this, "graph capture failed: %s", cudaGetErrorString(e));
@@ -775,6 +787,10 @@ struct Batch : lbs_batch {
 
     int step(int nsteps) override {
         if (nsteps <= 0) return LBS_OK;
+        if (!ready) {
+            berr(this, "no work lists: the last change of tiles or active instances failed");
+            return LBS_ECUDA;
+        }
         if (!use_graph) {
             for (int k = 0; k < nsteps; k++) {
                 int r = enqueue_step(stream, false);
@@ -803,7 +819,6 @@ struct Batch : lbs_batch {
     // each cost a synchronisation and a copy an instance, 40 ms for reading the
     // fields of 64).
     int collect() {
-        std::vector<int> set(n);
         kb_status<R><<<(n + 127) / 128, 128, 0, stream>>>(d_insts, n, d_status);
         BCK(cudaGetLastError());
         BCK(cudaMemcpyAsync(set.data(), d_status, n * sizeof(int), cudaMemcpyDeviceToHost, stream));
@@ -847,7 +862,7 @@ struct Batch : lbs_batch {
             berr(this, "instance %d of %d", k, n);
             return LBS_EINVAL;
         }
-        if (act[k] == (on ? 1 : 0)) return LBS_OK;
+        if (act[k] == (on ? 1 : 0) && ready) return LBS_OK;
         act[k] = on ? 1 : 0;
         return set_tiles(tx, ty, sv);
     }
@@ -908,6 +923,17 @@ struct Batch : lbs_batch {
     }
 };
 
+// f(), with the one exception that the lists' host memory may raise as a status
+template <typename F>
+int guarded(lbs_batch *b, F &&f) {
+    try {
+        return f();
+    } catch (const std::bad_alloc &) {
+        berr(b, "out of host memory");
+        return LBS_ENOMEM;
+    }
+}
+
 int check_batch(const lbs_params *p, int n, int storage, char *err, size_t len) {
     if (!p || n < 1) {
         snprintf(err, len, "a batch needs at least one instance");
@@ -958,12 +984,14 @@ int lbs_batch_create(const lbs_params *p, int n, int storage, void *stream, void
     *out = b;
     int r = check_batch(p, n, storage, b->err, sizeof(b->err));
     if (r) return r;
-    switch (storage) {
-    case LBS_F64: return ((Batch<double, double> *)b)->create(p, n, storage, stream, workspace, workspace_bytes);
-    case LBS_F32: return ((Batch<float, float> *)b)->create(p, n, storage, stream, workspace, workspace_bytes);
-    case LBS_F16: return ((Batch<float, __half> *)b)->create(p, n, storage, stream, workspace, workspace_bytes);
-    default: return ((Batch<float, __nv_bfloat16> *)b)->create(p, n, storage, stream, workspace, workspace_bytes);
-    }
+    return guarded(b, [&]() -> int {
+        switch (storage) {
+        case LBS_F64: return ((Batch<double, double> *)b)->create(p, n, storage, stream, workspace, workspace_bytes);
+        case LBS_F32: return ((Batch<float, float> *)b)->create(p, n, storage, stream, workspace, workspace_bytes);
+        case LBS_F16: return ((Batch<float, __half> *)b)->create(p, n, storage, stream, workspace, workspace_bytes);
+        default: return ((Batch<float, __nv_bfloat16> *)b)->create(p, n, storage, stream, workspace, workspace_bytes);
+        }
+    });
 }
 
 int lbs_batch_init_fields(lbs_batch *b, int k, const double *phi, const double *psi,
@@ -974,7 +1002,7 @@ int lbs_batch_init_fields(lbs_batch *b, int k, const double *phi, const double *
 
 int lbs_batch_set_tiles(lbs_batch *b, int tx, int ty, int sor_tile) {
     if (!b) return LBS_EINVAL;
-    return b->set_tiles(tx, ty, sor_tile);
+    return guarded(b, [&] { return b->set_tiles(tx, ty, sor_tile); });
 }
 
 int lbs_batch_step(lbs_batch *b, int n) {
@@ -1017,7 +1045,7 @@ int lbs_batch_status(lbs_batch *b, int *status) {
 
 int lbs_batch_set_active(lbs_batch *b, int k, int active) {
     if (!b) return LBS_EINVAL;
-    return b->set_active(k, active);
+    return guarded(b, [&] { return b->set_active(k, active); });
 }
 
 void lbs_batch_destroy(lbs_batch *b) {
