@@ -334,8 +334,9 @@ const char *lbs_last_error(const lbs_ctx *c);
  * Eotvos / Biot numbers, confinement; transport on) advanced together.
  * In FP32 arithmetic the step up to the moments of t+1 is one launch an
  * instance, side by side on streams of the batch between two events of its
- * own, and the solves of all instances are one cooperative launch where their
- * tiles fit the chip.  Other phases (and FP64) are one launch for the whole
+ * own (up to 16 instances, or 2^14 cells an instance on average), and the solves
+ * of all instances are one cooperative launch where their tiles fit the chip.
+ * Other phases (and many small instances, and FP64) are one launch for the whole
  * batch: a grid of (SM count x resident blocks) blocks walks a work list of
  * (instance, tile) items, and the SOR rounds run in one CUDA-graph WHILE loop.
  * Each instance has its own round counter and convergence test (Sec. 2.2

@@ -2,13 +2,14 @@
 // the coupled step: different grids, Eotvos and Biot numbers, confinement)
 // advanced together.
 //
-// In FP32 arithmetic everything up to the moments of t+1 is the fused step, one
-// launch an instance, side by side (kb_fused2).  Every other phase is one launch
-// for the whole batch: a grid of (SM count x resident blocks) blocks walks a
-// work list of (instance, tile) items, copies the instance's descriptor into
-// shared memory when the instance changes and runs the same per-cell bodies as
-// the single-instance kernels; FP64, bound by its arithmetic, of which a tile's
-// halo would be a quarter more, takes all phases that way.  The SOR rounds of
+// In FP32 arithmetic, unless the instances are many and small (Batch::fuse),
+// everything up to the moments of t+1 is the fused step, one launch an instance,
+// side by side (kb_fused2).  Every other phase is one launch for the whole batch: a
+// grid of (SM count x resident blocks) blocks walks a work list of (instance,
+// tile) items, copies the instance's descriptor into shared memory when the
+// instance changes and runs the same per-cell bodies as the single-instance
+// kernels; FP64, bound by its arithmetic, of which a tile's halo would be a
+// quarter more, takes all phases that way.  The SOR rounds of
 // all instances share one WHILE node: each instance keeps its own round
 // counter, convergence test and ping-pong parity, a converged instance's tiles
 // skip the remaining rounds, and the loop ends when no instance is still
@@ -44,7 +45,8 @@ struct BatchCtl {
     int active;           // instances still iterating in the current solve
 };
 
-enum { OP_FORCE, OP_FDCOLLIDE, OP_STREAM, OP_GRAD, OP_SCALE, NOPS };
+// OP_FDCOLLIDE_G: also leaves the solve's starting guess in psi2, C2 (kb_solve2)
+enum { OP_FORCE, OP_FDCOLLIDE, OP_STREAM, OP_GRAD, OP_SCALE, OP_FDCOLLIDE_G, NOPS };
 
 // copy descriptor k into shared memory (all threads; uniform) and return
 // whether the instance is alive (an instance whose total went non-finite is
@@ -80,13 +82,27 @@ __global__ void kb_cells2(const Inst<R> *__restrict__ insts, const WorkItem *__r
         const int x = it.x0 + threadIdx.x, y = it.y0 + threadIdx.y;
         if (OP == OP_FORCE)
             force2_cell(sI, x, y);
-        else if (OP == OP_FDCOLLIDE) {
+        else if (OP == OP_FDCOLLIDE || OP == OP_FDCOLLIDE_G) {
             // (the explicit surfactant terms and the collision in one pass)
             fd2_cell(sI, x, y, nullptr, nullptr);
             collide2_cell<R, P>(sI, x, y);
+            if (OP == OP_FDCOLLIDE_G && x < sI.nx && y < sI.ny) {
+                // (2 x^n - x^(n-1), see sor_guess; neighbours read psi, C, so
+                // the guess goes to the second buffers)
+                const long long c = (long long)y * sI.pitch + x;
+                const R p = sI.psi[c], q = sI.C[c];
+                sI.psi2[c] = R(2) * p - sI.psip[c];
+                sI.C2[c] = R(2) * q - sI.Cp[c];
+                sI.psip[c] = p;
+                sI.Cp[c] = q;
+            }
         }
-        else if (OP == OP_STREAM)
+        else if (OP == OP_STREAM) {
+            // (kb_solve2's barrier of this instance starts from a clear count)
+            if (it.x0 == 0 && it.y0 == 0 && threadIdx.x == 0 && threadIdx.y == 0)
+                sI.ctl->bar_count = 0;
             stream2_cell<R, P>(sI, x, y);
+        }
         else if (OP == OP_GRAD) {
             // (after the fused step the moments of t+1 are in the next set and
             // the starting guess is made)
@@ -320,9 +336,8 @@ struct Batch : lbs_batch {
     WorkItem *d_cells = nullptr, *d_sor = nullptr, *d_surf = nullptr;
     // kb_fused2: its tile (16 x 8 or 32 x 16), the instances' descriptors, and
     // the streams of the launches beside the batch's own
-    static constexpr bool kFused = sizeof(R) == 4;
     static constexpr int kSide = 7;
-    bool fused_small = false;
+    bool fused = false, fused_small = false;
     std::vector<Inst<R>> insts;
     cudaStream_t side[kSide] = {};
     cudaEvent_t fork = nullptr, joined[kSide] = {};
@@ -405,6 +420,7 @@ struct Batch : lbs_batch {
             BCK(cudaMalloc(&ws, total));
             own_ws = true;
         }
+        fused = fuse(p, n);
         std::vector<Inst<R>> &h = insts;
         h.resize(n);
         for (int k = 0; k < n; k++) {
@@ -423,10 +439,9 @@ struct Batch : lbs_batch {
                 berr(this, "internal: descriptor size mismatch");
                 return LBS_EINVAL;
             }
-            // FP64 runs the separate per-cell kernels: populations and moments
-            // return to set 0 every step and the SOR starting guess sits in
-            // psi, C; the fused step keeps them as a solver of its own does
-            if (!kFused) c->impl->set_batch_member();
+            // with the per-cell kernels populations and moments return to set 0
+            // every step; the fused step keeps them as a solver of its own does
+            if (!fused) c->impl->set_batch_member();
             std::memcpy(&h[k], c->impl->inst(), sizeof(Inst<R>));
             if (p[k].sor_max_iter > max_iter) max_iter = p[k].sor_max_iter;
         }
@@ -446,7 +461,7 @@ struct Batch : lbs_batch {
             BCK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)sor_smem<R>(v)));
         }
-        if constexpr (kFused) {
+        if (fused) {
             BCK(cudaFuncSetAttribute((void *)kb_fused2<R, P, 32, 16>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)Fuse2<R, 32, 16>::bytes()));
@@ -462,6 +477,21 @@ struct Batch : lbs_batch {
         return set_tiles(32, 8, 0);
     }
 
+    // whether the step up to the moments of t+1 is kb_fused2 (FP32 arithmetic): a
+    // launch an instance, eight side by side, costs 2.5 us an instance however
+    // small; the three cell phases take 0.2 ns a cell, the fused step 0.15.  Fused
+    // from 2^14 cells an instance on average; and up to 16 instances, where it
+    // costs the smallest ones 17 us a step at most (up to 8 nothing), because each
+    // then has the bits of a context of its own, which the phases, compiled
+    // apart, have not.  Steps of 64 instances, phases against fused, FP32: 32 x 48
+    // 56 and 171 us, 64 x 128 161 and 231, 64 x 200 246 and 285, 96 x 200 383
+    // and 366, 128 x 256 661 and 550 (FP16 alike).
+    static bool fuse(const lbs_params *p, int n) {
+        if (sizeof(R) != 4) return false;
+        long long cells = 0;
+        for (int k = 0; k < n; k++) cells += (long long)p[k].nx * p[k].ny;
+        return n <= 16 || cells >= ((long long)n << 14);
+    }
     template <int TX, int TY>
     long long fused_tiles() const {
         long long t = 0;
@@ -649,17 +679,11 @@ struct Batch : lbs_batch {
         n_surf = (int)surf.size();
         BCK(cudaMemcpy(d_act, act.data(), n * sizeof(int), cudaMemcpyHostToDevice));
         const int th = tx * ty;
-        const void *fk[NOPS] = {nullptr, nullptr, nullptr, (void *)kb_cells2<R, P, OP_GRAD>,
-                                (void *)kb_cells2<R, P, OP_SCALE>};
-        if constexpr (!kFused) {
-            fk[OP_FORCE] = (void *)kb_cells2<R, P, OP_FORCE>;
-            fk[OP_FDCOLLIDE] = (void *)kb_cells2<R, P, OP_FDCOLLIDE>;
-            fk[OP_STREAM] = (void *)kb_cells2<R, P, OP_STREAM>;
-        } else {
-            set_fused();
-        }
-        for (int o = 0; o < NOPS; o++)
-            if (fk[o]) g_cells[o] = persistent_grid(fk[o], th, 0, n_cells);
+        if (fused) set_fused();
+        const void *fk[NOPS] = {(void *)kb_cells2<R, P, OP_FORCE>, (void *)kb_cells2<R, P, OP_FDCOLLIDE>,
+                             (void *)kb_cells2<R, P, OP_STREAM>, (void *)kb_cells2<R, P, OP_GRAD>,
+                             (void *)kb_cells2<R, P, OP_SCALE>, (void *)kb_cells2<R, P, OP_FDCOLLIDE_G>};
+        for (int o = 0; o < NOPS; o++) g_cells[o] = persistent_grid(fk[o], th, 0, n_cells);
         g_sor = persistent_grid(sor_kernel(sizeof(R) == 8, sv), sor_vbs(sv), sor_smem<R>(sv), n_sor);
         g_surf = persistent_grid((void *)kb_surf2<R, kSurfBS>, kSurfBS, 0, n_surf);
         int rg = set_gang();
@@ -684,14 +708,19 @@ struct Batch : lbs_batch {
     // the launches of one step of the whole batch
     int enqueue_step(cudaStream_t s, bool capturing) {
         const dim3 blk(tx, ty, 1);
-        if constexpr (kFused) {
+        if (fused) {
             int r = enqueue_fused(s);
             if (r) return r;
         } else {
             kb_cells2<R, P, OP_FORCE><<<g_cells[OP_FORCE], blk, 0, s>>>(d_insts, d_cells, n_cells);
-            kb_cells2<R, P, OP_FDCOLLIDE><<<g_cells[OP_FDCOLLIDE], blk, 0, s>>>(d_insts, d_cells,
-                                                                              n_cells);
+            if (gang.fn)
+                kb_cells2<R, P, OP_FDCOLLIDE_G><<<g_cells[OP_FDCOLLIDE_G], blk, 0, s>>>(
+                    d_insts, d_cells, n_cells);
+            else
+                kb_cells2<R, P, OP_FDCOLLIDE><<<g_cells[OP_FDCOLLIDE], blk, 0, s>>>(d_insts, d_cells,
+                                                                                  n_cells);
             kb_cells2<R, P, OP_STREAM><<<g_cells[OP_STREAM], blk, 0, s>>>(d_insts, d_cells, n_cells);
+            BCK(cudaGetLastError());
         }
         if (gang.fn) {
             cudaLaunchConfig_t cfg = {};
@@ -897,13 +926,13 @@ struct Batch : lbs_batch {
         return LBS_OK;
     }
 
-    // launches of one step: the fused steps and kb_solve2; or the fused steps
-    // (FP64: 3 cell phases), the gradient, the SOR opener, the rounds of the slowest
+    // launches of one step: the fused steps or 3 cell phases, and kb_solve2 or the
+    // gradient, the SOR opener, the rounds of the slowest
     // instance at the last diagnostics, the total and the rescale
     int kernel_count() const override {
         int live = 0;
         for (int k = 0; k < n; k++) live += act[k];
-        return (kFused ? live : 3) + (gang.fn ? 1 : 4 + last_rounds);
+        return (fused ? live : 3) + (gang.fn ? 1 : 4 + last_rounds);
     }
 
     int set_sor_wait_limit(long long p) override {
