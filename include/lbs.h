@@ -287,7 +287,8 @@ int lbs_set_sor_tile(lbs_ctx *c, int variant);
  * orders, so FP32 results agree to rounding.  3D contexts with SOR variant 0 in
  * FP32 arithmetic: every sweep of a solve in one cooperative launch (on) or the
  * half-sweeps as launches of their own (off): the same iterates.  FP64 2D
- * grids of more tiles than SMs are swept a launch a round either way.  A
+ * grids of more tiles than SMs are swept a launch a round, which is faster,
+ * unless this call asks for one launch.  A
  * barrier that waits too long (about a second) reports LBS_ETIMEOUT.  Errors:
  * LBS_EINVAL (no context), LBS_ECUDA. */
 int lbs_set_sor_persistent(lbs_ctx *c, int on);

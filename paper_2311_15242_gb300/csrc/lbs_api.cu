@@ -449,11 +449,13 @@ struct Solver : Base {
             const long long tiles = (long long)sor_grid.x * sor_grid.y;
             const long long resident = (long long)per_sm * sms;
             coop_blocks = (int)(tiles < resident ? tiles : resident);
-            // (FP64 only while every tile has an SM: beyond, a launch a round
-            // spreads them better than blocks that wait for each other; SOR,
-            // gradient and total at 250 x 250, 128 tiles: 186 us in one launch,
-            // 217 in several; 300 x 300, 190: 287 and 278; 400 x 400, 325: 520 and 425)
-            coop_ok = coop && coop_blocks > 0 && (sizeof(R) == 4 || s2 == kSorSmall || tiles <= sms);
+            coop_ok = coop && coop_blocks > 0;
+            // (FP64, unless asked for: only while every tile has an SM.  Beyond, a
+            // launch a round spreads them better than blocks that wait for each
+            // other; SOR, gradient and total at 250 x 250, 128 tiles: 186 us in one
+            // launch, 217 in several; 300 x 300, 190: 287 and 278; 400 x 400, 325:
+            // 520 and 425)
+            coop_slow = sizeof(R) == 8 && s2 != kSorSmall && tiles > sms;
             set_solve(coop ? sms : 0);
         }
     }
@@ -503,8 +505,12 @@ struct Solver : Base {
     }
     int coop_blocks = 0;  // blocks of the one-launch form
     bool coop_ok = false;  // the one-launch SOR applies to this grid and variant
-    bool coop_on = true;   // and is wanted (lbs_set_sor_persistent)
-    bool use_coop() const { return D == 2 && coop_ok && coop_on; }
+    bool coop_slow = false;   // a launch a round is faster
+    bool coop_on = true;      // and is wanted (lbs_set_sor_persistent),
+    bool coop_asked = false;  // by the caller
+    bool use_coop() const {
+        return D == 2 && coop_ok && coop_on && (coop_asked || !coop_slow);
+    }
     long long coop_polls = kBarrierPolls;  // the barrier's wait limit
     int set_sor_wait_limit(long long polls) override {
         if (polls < 0) {
@@ -523,7 +529,7 @@ struct Solver : Base {
     }
     int set_sor_persistent(int on) override {
         CK(cudaStreamSynchronize(ctx->stream));
-        coop_on = on != 0;
+        coop_on = coop_asked = on != 0;
         if (D == 3) set_sor_grid();
         if (gexec) {
             CK(cudaGraphExecDestroy(gexec));
