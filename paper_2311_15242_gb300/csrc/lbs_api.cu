@@ -157,9 +157,10 @@ FusedTile fused_tile() {
 // tile, one a SM: 16 x 8 wins up to one 32 x 16 tile an SM (128 x 128, 32
 // tiles: 309 -> 106 us; 250 x 250, 128: 311 -> 268; 300 x 400, 250: 428 -> 438).
 // FP32 is bound by the latency of a tile's phases, which a smaller tile
-// shortens while each still has an SM of its own, up to half the SMs (64 x
-// 517, 66 tiles: 22.1 -> 17.9 us; 64 x 1024, 128: 21.4 -> 19.9; 96 x 700,
-// 132: 20.0 -> 20.3; 128 x 1000, 252: 24.9 -> 25.9).
+// shortens until its four times as many blocks fill the SMs.  Gain and loss meet
+// between 66 large tiles and 132 (64 x 517, 66: 22.1 -> 17.9 us; 64 x 1024, 128:
+// 21.4 -> 19.9; 96 x 700, 132: 20.0 -> 20.3; 128 x 1000, 252: 24.9 -> 25.9); the
+// line at half as many as SMs is on the safe side of that.
 template <typename R, typename P>
 FusedTile fused_tile_for(int nx, int ny, int sms) {
     const FusedTile big = fused_tile<R, P, 32, 16>();

@@ -26,9 +26,6 @@
 
 namespace lbs {
 
-template <typename R>
-__device__ __forceinline__ R cs2_lattice() { return R(1) / R(3); }
-
 // shift of direction i for a cell with the given flag
 template <typename R>
 __device__ __forceinline__ R shift_of(const Inst<R> &I, int i, int flag) {
@@ -598,23 +595,6 @@ __device__ __forceinline__ void collide2_cell(const Inst<R> &I, int x, int y) {
     I.gflag[c] = (uint8_t)fl;
 }
 
-// the explicit surfactant terms and the collision in one pass: both read
-// only what k_force and the previous stream / grad kernels wrote, and they
-// write disjoint fields
-template <typename R, typename P>
-__global__ void __launch_bounds__(256, 4) k_fdcollide2(Inst<R> I) {
-    pdl_wait();
-    pdl_trigger();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (I.transport) fd2_cell(I, x, y, nullptr, nullptr);
-    collide2_cell<R, P>(I, x, y);
-}
-
-template <typename R, typename P>
-__global__ void k_collide2(Inst<R> I) {
-    collide2_cell<R, P>(I, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y);
-}
-
 // ---------------------------------------------------------------------------
 // k_stream: f_i(x, t+1) = f_i^post(x - e_i) (Eq. 13, pull form); a link that
 // crosses a wall is reflected (half-way bounce-back), a moving wall adds
@@ -774,13 +754,6 @@ __device__ __forceinline__ void stream2_cell(const Inst<R> &I, int x, int y) {
     I.fM0[c] = fM[0];
     I.flag[c] = (uint8_t)fl;
     store_moments(I, c, fT, fM, fl);
-}
-
-template <typename R, typename P>
-__global__ void k_stream2(Inst<R> I) {
-    pdl_wait();
-    pdl_trigger();
-    stream2_cell<R, P>(I, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y);
 }
 
 // ---------------------------------------------------------------------------

@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_collide3(Inst<R
         const R fr = fdiv(rmin, rdag);
         const R sg = fl ? R(-1) : R(1);
         // moving populations as stored; the rest populations close the cell's
-        // total and minority mass on the pre-collision values (see k_collide2)
+        // total and minority mass on the pre-collision values (see collide2_cell)
         CSum<R> sT, sM;
         const unsigned int rk = rest_key(c, rest_salt(0, I.ctl->step)), rs = pop_seed(rk);
 #pragma unroll
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_collide3(Inst<R
 }
 
 // streaming (Eq. 13, pull), half-way bounce-back with moving walls, moments
-// at t+1 (see k_stream2).  Bound by the wait for the 38 populations a cell
+// at t+1 (see stream2_cell).  Bound by the wait for the 38 populations a cell
 // pulls: 4 blocks an SM (64 registers; 5 spill in the fast path and 3 wait
 // longer), which took the general path's second copy of them out of the fast
 // one.  100 cubed FP32, mirror planes: 107 -> 84 us (half of the copy bandwidth),
