@@ -143,8 +143,9 @@ __global__ void k_moments3(Inst<R> I) {
 // although a cell then reads 2.1 slots instead of 1.8); FP64 takes 2 to stay
 // within 48 KB.  Measured in FP32 at 100 cubed: gradient 34 -> 25 us, force 57
 // -> 29, collision 129 -> 103; at 256 x 128 x 128 with BF16 populations 88 -> 66,
-// 226 -> 165, 406 -> 304.  What is left is the wait for memory: 25 to 60 % of
-// the issue slots are used, 20 to 55 % of the copy bandwidth.
+// 226 -> 165, 406 -> 304.  What is left is the wait for memory and instruction issue
+// side by side: at 256 x 128 x 64, BF16, the three use 44, 68 and 72 % of the
+// issue slots and 32 % of the DRAM's peak each.
 // ---------------------------------------------------------------------------
 template <typename R>
 struct Tile3 {

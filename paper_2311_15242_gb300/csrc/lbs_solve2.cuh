@@ -29,8 +29,8 @@
 // 1024 (8 sweeps, FP32) k_sorfuse2 (32 x 16 tiles, 2 sweeps a round: twelve 8-byte
 // shared accesses and about 60 instructions an update, FP64 in every thread's
 // reductions, a grid barrier of 512 blocks five times) takes 65 us, this form
-// 34 with 145 blocks (27 us of it in the kernel: 9 until the first sweep, 2 x
-// 4.4 for 4 sweeps, 2 x 5 from publishing the tile to the decision); at 64 x 517
+// 34 with 145 blocks (about 9 until the first sweep, 2 x 4.4 for 4 sweeps, 2 x 5
+// from publishing the tile to the decision; 36 % of the issue slots); at 64 x 517
 // (33 blocks, 6 sweeps) 53 -> 33 us, at 241 x 1011 (odd periodic axis) 90 -> 41.
 #pragma once
 
