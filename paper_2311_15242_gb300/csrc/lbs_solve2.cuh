@@ -125,7 +125,6 @@ struct SolveSmem {
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
     return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
 }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 shfl_up2(float2 v) {
     return make_float2(__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1));
 }
@@ -136,18 +135,28 @@ __device__ __forceinline__ float2 shfl_down2(float2 v) {
 __device__ __forceinline__ float warp_max_pos(float v) {
     return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
 }
-// sums of the compensated sums hi + lo of groups of 2 o lanes, for two rounds
-// side by side (the halves' order does not matter: every lane gets the same)
-__device__ __forceinline__ void lane_sums(float2 &hi, float2 &lo, int o) {
+// a sum as three floats, hi + lo + rest: adding another keeps the rounding errors
+// of hi and of lo, so that some 70 bits count
+__device__ __forceinline__ void add3(float &hi, float &lo, float &rest, float h, float l, float r) {
+    float e, el, ee;
+    hi = two_sum(hi, h, e);
+    lo = two_sum(two_sum(lo, l, el), e, ee);
+    rest = (rest + r) + (el + ee);
+}
+// the warp's sums of NR rounds side by side, in every lane
+template <int NR>
+__device__ __forceinline__ void lane_sum3(float (&hi)[NR], float (&lo)[NR], float (&rest)[NR]) {
 #pragma unroll 1
-    for (; o > 0; o >>= 1) {
-        const float2 h = make_float2(__shfl_xor_sync(0xffffffffu, hi.x, o),
-                                     __shfl_xor_sync(0xffffffffu, hi.y, o));
-        const float2 g = make_float2(__shfl_xor_sync(0xffffffffu, lo.x, o),
-                                     __shfl_xor_sync(0xffffffffu, lo.y, o));
-        float2 e;
-        hi = make_float2(two_sum(hi.x, h.x, e.x), two_sum(hi.y, h.y, e.y));
-        lo = add2(add2(lo, g), e);
+    for (int o = 16; o > 0; o >>= 1) {
+        float h[NR], l[NR], r[NR];
+#pragma unroll
+        for (int n = 0; n < NR; n++) {
+            h[n] = __shfl_xor_sync(0xffffffffu, hi[n], o);
+            l[n] = __shfl_xor_sync(0xffffffffu, lo[n], o);
+            r[n] = __shfl_xor_sync(0xffffffffu, rest[n], o);
+        }
+#pragma unroll
+        for (int n = 0; n < NR; n++) add3(hi[n], lo[n], rest[n], h[n], l[n], r[n]);
     }
 }
 // a plane's element at a byte offset (32 bits: one register an address)
@@ -169,8 +178,9 @@ __device__ __forceinline__ bool solve_converged(const float *m, float before, bo
 
 // tile (bx, by), block `blk` of the nb of grid I's gang.  FP64 runs at 1/64 of
 // FP32's rate, so the surfactant is summed in compensated FP32 pairs within a
-// warp (256 cells; exact to about 48 bits) and in FP64 across warps and blocks,
-// the latter once, when the round that ends the solve is known.  The code is kept short (loops over
+// thread (8 cells), in three floats a sum within a warp (pairs there were off
+// by four times FP64's error on a grid of 11 warps) and in FP64 across warps and
+// blocks, the latter once, when the round that ends the solve is known.  The code is kept short (loops over
 // a thread's cells are rolled where the cells can pass through shared memory): with
 // little work a thread, the time of a launch is that of fetching its
 // instructions; unrolled over the eight cells it had 144 KB of code and took
@@ -188,7 +198,8 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
     float2 *Fr = Xs;
     float2 *Sn = (float2 *)(smem + 2 * S::w_bytes + S::x_bytes);
     __shared__ __align__(16) float redm[NW][8], redb[8][8];
-    __shared__ float4 reds[NW];  // a warp's sums of two rounds (hi, hi, lo, lo)
+    __shared__ float strip[3][kSolveThreads];  // the threads' sums of the first round of two
+    __shared__ float reds[3][2][NW];           // the warps' sums of the rounds
     __shared__ double2 sums[kSolveMaxBlocks];  // the blocks' sums of the last phase
     __shared__ struct {
         double M0;     // the conserved total
@@ -420,7 +431,7 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
     unsigned int bt = 0;
 #pragma unroll 1
     for (int ph = 0;; ph++) {
-        float2 tsum = make_float2(0.f, 0.f), tsum1 = tsum;  // (hi, lo) of the rounds
+        float th = 0.f, tl = 0.f, tr = 0.f;  // the thread's sum, of the last round
 #pragma unroll 1
         for (int n = 0; n < NR; n++) {
             float2 md = make_float2(0.f, 0.f), mx = make_float2(0.f, 0.f);
@@ -533,11 +544,15 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
                     comp_add_prod(hi.y, lo.y, wt.y, X[r][q].y);
                     if (n + 1 < NR) Sn[slot(r, q)] = X[r][q];
                 }
-            float e;
-            hi.x = two_sum(hi.x, hi.y, e);
-            lo.x = (lo.x + lo.y) + e;
-            if (n == 0) tsum = make_float2(hi.x, lo.x);
-            if (n == 1) tsum1 = make_float2(hi.x, lo.x);
+            th = hi.x;
+            tl = lo.x;
+            tr = 0.f;
+            add3(th, tl, tr, hi.y, lo.y, 0.f);
+            if (n + 1 < NR) {
+                strip[0][tid] = th;
+                strip[1][tid] = tl;
+                strip[2][tid] = tr;
+            }
             md.x = warp_max_pos(md.x);
             md.y = warp_max_pos(md.y);
             mx.x = warp_max_pos(mx.x);
@@ -559,9 +574,21 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
             }
         }
         {
-            float2 hi = make_float2(tsum.x, tsum1.x), lo = make_float2(tsum.y, tsum1.y);
-            lane_sums(hi, lo, 16);
-            if (l == 0) reds[w] = make_float4(hi.x, hi.y, lo.x, lo.y);
+            float sh[NR], sl[NR], sr[NR];
+#pragma unroll
+            for (int n = 0; n < NR; n++) {
+                sh[n] = n + 1 < NR ? strip[0][tid] : th;
+                sl[n] = n + 1 < NR ? strip[1][tid] : tl;
+                sr[n] = n + 1 < NR ? strip[2][tid] : tr;
+            }
+            if (live) lane_sum3<NR>(sh, sl, sr);  // (else zeros)
+            if (l == 0)
+#pragma unroll
+                for (int n = 0; n < NR; n++) {
+                    reds[0][n][w] = sh[n];
+                    reds[1][n][w] = sl[n];
+                    reds[2][n][w] = sr[n];
+                }
         }
         __syncthreads();
         // the tile's record, the grid barrier (see grid_barrier), everybody's
@@ -574,9 +601,11 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
             float v = fmaxf(fmaxf(p[0], p[8]), fmaxf(p[16], p[24]));
             v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
             v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 16));
-            const float4 u = reds[l & (NW - 1)];
-            double2 s = make_double2(double(u.x) + double(u.z), 0.0);
-            if (NR > 1) s.y = double(u.y) + double(u.w);
+            auto warp_total = [&](int n) {
+                const int k = l & (NW - 1);
+                return (double(reds[0][n][k]) + double(reds[1][n][k])) + double(reds[2][n][k]);
+            };
+            double2 s = make_double2(warp_total(0), NR > 1 ? warp_total(NR - 1) : 0.0);
 #pragma unroll
             for (int o = NW / 2; o > 0; o >>= 1) {
                 s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
