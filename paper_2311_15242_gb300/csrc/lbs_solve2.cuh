@@ -11,8 +11,8 @@
 // faces and inverse diagonals of their rows (the right-hand sides wait in shared
 // memory for want of registers).  An update is that of sor_tile2_cb, operation by
 // operation and rounding by rounding, so the results are its own to the bit
-// (but where the totals, summed in other orders, round the rescale step apart:
-// some four steps in a million).  The x-neighbour outside the pair comes from the
+// (but where the totals, summed in other orders, differ by an ulp and a cell's
+// rescale rounds apart: once in about 3 10^8 cells times steps).  The x-neighbour outside the pair comes from the
 // adjacent lane by shuffle; of the y-neighbours only those in another warp's rows
 // go through shared memory.  A half-sweep
 // updates one cell of every pair, spreads the error of the stale region edge

@@ -35,3 +35,14 @@ def test_scatter_does_not_choose_a_cell_tile(tmp_path):
     r = AT.tune(FakeBatch(), [128], timer=lambda b: next(scatter),
                 cache_path=str(tmp_path / "tiles.json"))
     assert (r["tx"], r["ty"], r["sor"]) == (*AT.CELL_TILES[0], 0)
+
+
+def test_a_run_that_settles_does_not_choose_a_cell_tile(tmp_path):
+    """The first steps of a run take more solver rounds, whatever the tile."""
+    n = [0]
+
+    def settling(b):
+        n[0] += 1
+        return 1.0 + 0.5 / n[0]
+    r = AT.tune(FakeBatch(), [128], timer=settling, cache_path=str(tmp_path / "tiles.json"))
+    assert (r["tx"], r["ty"]) == AT.CELL_TILES[0]
