@@ -52,6 +52,7 @@ struct SolveGeom {
 constexpr int kSolveRegion = 64;   // largest side of a region
 constexpr int kSolveThreads = 512;
 constexpr int kSolveMaxBlocks = 256;  // blocks of a gang at most
+constexpr int kSolveFine = 32;        // blocks from which a warp's sums are pairs
 
 // what a block leaves for the others at a grid barrier: for each of at most
 // two rounds the largest |d psi|, |d C|, |psi|, |C| of its last sweep and the
@@ -143,11 +144,35 @@ __device__ __forceinline__ void add3(float &hi, float &lo, float &rest, float h,
     lo = two_sum(two_sum(lo, l, el), e, ee);
     rest = (rest + r) + (el + ee);
 }
-// the warp's sums of NR rounds side by side, in every lane
+// the sums of groups of 2 `from` lanes, of NR rounds side by side, in every lane; not
+// `fine`: as pairs (48 bits)
 template <int NR>
-__device__ __forceinline__ void lane_sum3(float (&hi)[NR], float (&lo)[NR], float (&rest)[NR]) {
+__device__ __forceinline__ void lane_sum3(float (&hi)[NR], float (&lo)[NR], float (&rest)[NR],
+                                          bool fine, int from = 16) {
+    if (!fine) {
+#pragma unroll
+        for (int n = 0; n < NR; n++) {
+            lo[n] += rest[n];
+            rest[n] = 0.f;
+        }
 #pragma unroll 1
-    for (int o = 16; o > 0; o >>= 1) {
+        for (int o = 16; o > 0; o >>= 1) {
+            float h[NR], l[NR], e;
+#pragma unroll
+            for (int n = 0; n < NR; n++) {
+                h[n] = __shfl_xor_sync(0xffffffffu, hi[n], o);
+                l[n] = __shfl_xor_sync(0xffffffffu, lo[n], o);
+            }
+#pragma unroll
+            for (int n = 0; n < NR; n++) {
+                hi[n] = two_sum(hi[n], h[n], e);
+                lo[n] = (lo[n] + l[n]) + e;
+            }
+        }
+        return;
+    }
+#pragma unroll 1
+    for (int o = from; o > 0; o >>= 1) {
         float h[NR], l[NR], r[NR];
 #pragma unroll
         for (int n = 0; n < NR; n++) {
@@ -178,9 +203,11 @@ __device__ __forceinline__ bool solve_converged(const float *m, float before, bo
 
 // tile (bx, by), block `blk` of the nb of grid I's gang.  FP64 runs at 1/64 of
 // FP32's rate, so the surfactant is summed in compensated FP32 pairs within a
-// thread (8 cells), in three floats a sum within a warp (pairs there were off
-// by four times FP64's error on a grid of 11 warps) and in FP64 across warps and
-// blocks, the latter once, when the round that ends the solve is known.  The code is kept short (loops over
+// thread (8 cells) and a warp (256; their errors average out over the warps, but
+// a gang of fewer than 32 blocks takes three floats a sum: of 11 warps, pairs
+// were off by four times FP64's error), in three floats across a block's warps (a
+// chain of FP64 adds there costs a step 1 us) and in FP64 across the blocks, once,
+// when the round that ends the solve is known.  The code is kept short (loops over
 // a thread's cells are rolled where the cells can pass through shared memory): with
 // little work a thread, the time of a launch is that of fetching its
 // instructions; unrolled over the eight cells it had 144 KB of code and took
@@ -581,7 +608,7 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
                 sl[n] = n + 1 < NR ? strip[1][tid] : tl;
                 sr[n] = n + 1 < NR ? strip[2][tid] : tr;
             }
-            if (live) lane_sum3<NR>(sh, sl, sr);  // (else zeros)
+            if (live) lane_sum3<NR>(sh, sl, sr, nb < kSolveFine);  // (else zeros)
             if (l == 0)
 #pragma unroll
                 for (int n = 0; n < NR; n++) {
@@ -601,16 +628,16 @@ __device__ __forceinline__ void solve2_tile(const Inst<float> &I, const SolveGeo
             float v = fmaxf(fmaxf(p[0], p[8]), fmaxf(p[16], p[24]));
             v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
             v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 16));
-            auto warp_total = [&](int n) {
-                const int k = l & (NW - 1);
-                return (double(reds[0][n][k]) + double(reds[1][n][k])) + double(reds[2][n][k]);
-            };
-            double2 s = make_double2(warp_total(0), NR > 1 ? warp_total(NR - 1) : 0.0);
+            float sh[NR], sl[NR], sr[NR];
 #pragma unroll
-            for (int o = NW / 2; o > 0; o >>= 1) {
-                s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-                if (NR > 1) s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+            for (int n = 0; n < NR; n++) {
+                sh[n] = reds[0][n][l & (NW - 1)];
+                sl[n] = reds[1][n][l & (NW - 1)];
+                sr[n] = reds[2][n][l & (NW - 1)];
             }
+            lane_sum3<NR>(sh, sl, sr, true, NW / 2);
+            auto whole = [&](int n) { return (double(sh[n]) + double(sl[n])) + double(sr[n]); };
+            const double2 s = make_double2(whole(0), NR > 1 ? whole(NR - 1) : 0.0);
             if (l < 8) recs[blk].m[l] = v;
             if (l == 0) recs[blk].sum = s;
             __syncwarp();
