@@ -1325,7 +1325,6 @@ __device__ __forceinline__ bool grid_barrier(Ctl *ctl, unsigned int nblocks,
     target += nblocks;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
         ok = barrier_arrive(ctl, target, max_looks);
         const volatile unsigned int *count = &ctl->bar_count;
         for (long long looks = 0; ok && *count < target;) {
