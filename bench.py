@@ -84,13 +84,13 @@ POP_BYTES = {"f64": 8, "f32": 4, "f16": 2, "bf16": 2}
 # six times the L2), which the 4096 x 4096 array's roofline scales by its
 # cells (the kernels' traffic grows with the cells).  Reported only while the
 # files that hold their device code (FUSED2_FILES) hash as below.
-TRAFFIC = {"kernel_sha": "290842b2b78c2c26",
+TRAFFIC = {"kernel_sha": "5cc4dea806af04bf",
            "bytes_per_cell": {"0": {"collide": 129.8, "sor": 24.3},
-                              "4": {"collide": 129.9, "sor": 24.3},
-                              "5": {"collide": 130.0, "sor": 24.3},
-                              "6": {"collide": 129.9, "sor": 24.3}},
+                              "4": {"collide": 129.8, "sor": 24.3},
+                              "5": {"collide": 129.9, "sor": 24.3},
+                              "6": {"collide": 129.8, "sor": 24.3}},
            "bytes_per_cell_hbm": {"4": {"collide": 243.8, "sor": 200.8},
-                                  "5": {"collide": 243.7, "sor": 200.3},
+                                  "5": {"collide": 243.8, "sor": 200.3},
                                   "6": {"collide": 243.8, "sor": 200.4}}}
 
 
